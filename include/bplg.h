@@ -21,7 +21,7 @@
  *   - Memory: the caller owns every buffer and every stream.  "device" buffers
  *     are CUDA global memory of the current device; "host" buffers are CPU
  *     memory.  Compute entry points never allocate on their hot path; the
- *     first FFT call on a device allocates the shared twiddle table (256 KB)
+ *     first FFT call on a device allocates the shared twiddle table (512 KB)
  *     once, synchronously, so it must not be the first call inside a stream
  *     capture.  The library keeps such per-device state (tables, scratch,
  *     kernel attributes) for the life of the process: do not use it on a
@@ -233,7 +233,7 @@ int bplg_fft_tc_batched(const void *in, void *out, int64_t n, int64_t batch, int
  * counterpart: this is a property of the library, not of the method.
  *
  * It calls no cudaMalloc, cudaFree or other allocating routine: its twiddle
- * table is a file-scope device array of 64 KB that every GPU loading the
+ * table is a file-scope device array of 128 KB that every GPU loading the
  * library holds until the process exits, so it accepts only n <= 4096 (larger
  * n returns BPLG_ERR_UNSUPPORTED_SIZE with a message).  On success nothing is
  * allocated; on failure the error message string may be.

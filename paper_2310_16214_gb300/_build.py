@@ -27,7 +27,7 @@ EXTREF_LIB = os.path.join(OUT_DIR, "libbplg_extref.so")
 
 GEN_DIR = os.path.join(OUT_DIR, "gen")
 NOALLOC_TABLE = os.path.join(GEN_DIR, "noalloc_twiddles.inc")
-NOALLOC_MAX_LOG = 12  # the no-alloc FFT entry point's table holds W_M^k for M <= 4096
+NOALLOC_MAX_LOG = 12  # the no-alloc FFT entry point's table holds the roots of unity of order M <= 4096
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
@@ -49,25 +49,31 @@ def _sincospi(t: float):
 
 def write_noalloc_table() -> str:
     """Write the static initializer of the no-alloc FFT entry point's twiddle
-    array: tw[M + k] = exp(-2 pi i k / M) for M = 2, 4, ..., 2^NOALLOC_MAX_LOG
-    (tw[0] = tw[1] = 1), in float64, rounded once to float32, as hexadecimal
+    array, for M = 2, 4, ..., 2^NOALLOC_MAX_LOG the two blocks of M entries
+    described in csrc/fft_common.cuh: W_M^e = exp(-2 pi i e / M) at [2 M + e]
+    and, for M >= 16, W_M^(r k) at [3 M + r M / 16 + k] (1 in the unused
+    places), in float64, rounded once to float32, as hexadecimal
     float literals.  The file is rewritten only when its text changes."""
     import struct
-    total = 2 << NOALLOC_MAX_LOG
+    total = 4 << NOALLOC_MAX_LOG
 
     def f32(v: float) -> str:
         r = struct.unpack("<f", struct.pack("<f", v))[0]  # round to nearest float32
         return (r.hex() if r != 0.0 else ("-0x0p+0" if math.copysign(1.0, r) < 0 else "0x0p+0")) + "f"
 
     import math
-    lines = ["// generated by _build.py: tw[M + k] = exp(-2 pi i k / M), M = 2 .. %d, float64 rounded to float32"
+    lines = ["// generated by _build.py: W_M^e at [2 M + e], stage blocks at [3 M ..], M = 2 .. %d, float64 rounded to float32"
              % (1 << NOALLOC_MAX_LOG)]
     for i in range(total):
-        if i < 2:
+        M = 1 << (i.bit_length() - 2) if i >= 4 else 1
+        k = i - 2 * M
+        if M < 2 or (k >= M and M < 16):
             c, s_ = 1.0, 0.0
         else:
-            M = 1 << (i.bit_length() - 1)
-            s_, c = _sincospi(-2.0 * (i - M) / M)
+            if k >= M:
+                r, kk = divmod(k - M, M // 16)
+                k = r * kk
+            s_, c = _sincospi(-2.0 * k / M)
         lines.append("{%s, %s}," % (f32(c), f32(s_)))
     text = "\n".join(lines) + "\n"
     os.makedirs(GEN_DIR, exist_ok=True)

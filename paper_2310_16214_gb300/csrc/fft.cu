@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(MAXT)
             const int Ns = 1 << logNs;
             const int k = j & (Ns - 1);
             if (logNs > 0) {
-                const float2 *twp = tw + (Ns << LR);
+                const float2 *twp = tw + tw_root(Ns << LR);
 #pragma unroll
                 for (int r = 1; r < R; ++r) {
                     float2 w = __ldg(twp + r * k);
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(MAXT)
                 const int Ns = 1 << logNs;
                 const int kk = j & (Ns - 1);
                 if (logNs > 0) {
-                    const float2 *twp = tw + (Ns << LR);
+                    const float2 *twp = tw + tw_root(Ns << LR);
 #pragma unroll
                     for (int r = 1; r < R; ++r) {
                         float2 w = __ldg(twp + r * kk);
@@ -520,19 +520,22 @@ __global__ void __launch_bounds__(MAXT)
     }
 }
 
-// Twiddle table: tw[M + k] = exp(-2 pi i k / M) for M = 2, 4, ..., 2^max_log,
-// computed in float64 and rounded once to float32.
+// Twiddle table (layout: tw_root and tw_stage16 in fft_common.cuh), computed
+// in float64 and rounded once to float32.
 __global__ void twiddle_init_kernel(float2 *tw, int max_log) {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    const int64_t total = int64_t(2) << max_log;
+    const int64_t total = tw_entries(max_log);
     if (i >= total) return;
-    if (i < 2) {
+    const int64_t M = i < 4 ? 1 : int64_t(1) << (62 - __clzll(static_cast<unsigned long long>(i)));
+    int64_t k = i - 2 * M;
+    if (M < 2 || (k >= M && M < 16)) {
         tw[i] = make_float2(1.f, 0.f);
         return;
     }
-    const int lm = 63 - __clzll(static_cast<unsigned long long>(i));
-    const int64_t M = int64_t(1) << lm;
-    const int64_t k = i - M;
+    if (k >= M) {  // stage block: W_M^(r k'), k' fastest
+        const int64_t q = k - M, ns = M / 16;
+        k = (q / ns) * (q % ns);
+    }
     double sn, cs;
     sincospi(-2.0 * static_cast<double>(k) / static_cast<double>(M), &sn, &cs);
     tw[i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
@@ -684,7 +687,7 @@ int twiddles_for_current_device(const void **tw) {
         *tw = it->second;
         return BPLG_OK;
     }
-    const int64_t total = int64_t(2) << kFftMaxLog;
+    const int64_t total = tw_entries(kFftMaxLog);
     float2 *p = nullptr;
     e = cudaMalloc(&p, total * sizeof(float2));
     if (e != cudaSuccess) return cuda_error(e, "twiddle table cudaMalloc");
@@ -782,7 +785,7 @@ int fft_device_status(int *flag, bool reset) {
 // trigger the implicit device synchronisation an allocation can cause, and
 // code whose allocations are only permitted during start-up.  For them the
 // twiddle table lives in the file-scope device array below, sized for
-// transforms of at most kNoAllocMaxN points (64 KB): every GPU that loads the
+// transforms of at most kNoAllocMaxN points (128 KB): every GPU that loads the
 // library holds it until the process exits.  The caller still provides the
 // input and output buffers.
 namespace bplg {
@@ -793,12 +796,12 @@ constexpr int kNoAllocMaxDevices = 64;
 
 }  // namespace bplg
 
-// W_M^k at [M + k] for M = 2 .. kNoAllocMaxN, as in the regular table.  The
+// The blocks of M = 2 .. kNoAllocMaxN, laid out as in the regular table.  The
 // values are part of the module image (a static initializer written at build
 // time from float64 values rounded once to float32), so the array is ready
 // as soon as the module is loaded on a device: no fill kernel, no wait, and a
 // module reloaded after cudaDeviceReset holds them again.
-static __device__ __align__(256) float2 g_noalloc_twiddles[2 * bplg::kNoAllocMaxN] = {
+static __device__ __align__(256) float2 g_noalloc_twiddles[bplg::tw_entries(bplg::kNoAllocMaxLog)] = {
 #include "noalloc_twiddles.inc"
 };
 

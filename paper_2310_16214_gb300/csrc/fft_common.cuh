@@ -31,6 +31,24 @@ __host__ __device__ constexpr float cos16(int k) {
 }
 __host__ __device__ constexpr float sin16(int k) { return cos16(k - 4); }
 
+// The twiddle table (one per device; the no-alloc entry point holds a shorter
+// one of the same layout).  For every M = 2, 4, .. the largest length there
+// are two blocks of M entries:
+//   [2 M + e]               W_M^e = exp(-2 pi i e / M), e < M;
+//   [3 M + r (M / 16) + k]  W_M^(r k), r < 16, k < M / 16 (M >= 16): the
+//                           twiddles of a radix-16 stage of stride Ns = M / 16
+//                           with the butterfly index k fastest.
+// In a radix-16 stage consecutive threads have consecutive k.  Read at W_M^(r k)
+// of the first block, a warp's 32 lanes lie 8 r bytes apart and one load
+// touches up to 2 r lines of 128 bytes; in the second block they are adjacent
+// (two lines).  Those loads were half of the L1 data-pipe work of the
+// 4096-point transform, whose pipe was 76 % busy.  Measured at 2^24 elements
+// on one GB300, first -> second layout: 1024 points 0.0487 -> 0.0468 ms, 4096
+// 0.0556 -> 0.0490, 8192 0.0736 -> 0.0632, 16384 0.0976 -> 0.0820.
+__host__ __device__ __forceinline__ constexpr int tw_root(int M) { return 2 * M; }
+__host__ __device__ __forceinline__ constexpr int tw_stage16(int M) { return 3 * M; }
+__host__ __device__ __forceinline__ constexpr int tw_entries(int max_log) { return 4 << max_log; }
+
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 w) {
@@ -200,10 +218,11 @@ __device__ __forceinline__ void fft_fixed_stages_st(float2 (&v)[R], float2 *buf2
         constexpr int LNS = O::LNS;
         if constexpr (LNS > 0) {
             const int k = j & ((1 << LNS) - 1);
-            const float2 *twk = tw + ((1 << LNS) << S::LR);
+            constexpr int M = (1 << LNS) << S::LR;
+            const float2 *twk = R == 16 ? tw + tw_stage16(M) + k : tw + tw_root(M);
 #pragma unroll
             for (int r = 1; r < R; ++r) {
-                float2 w = __ldg(twk + r * k);
+                float2 w = __ldg(twk + (R == 16 ? r << LNS : r * k));
                 if (DIR > 0) w.y = -w.y;
                 v[r] = cmul(v[r], w);
             }

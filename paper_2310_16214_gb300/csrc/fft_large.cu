@@ -50,7 +50,7 @@ constexpr int kFineLog = 12;          // fine twiddle table: W_n^j, j < 4096
 __device__ __forceinline__ float2 twiddle_n(const float2 *__restrict__ tw, const float2 *__restrict__ fine, int logn,
                                             uint32_t m, int dir) {
     const float2 lo = __ldg(fine + (m & ((1u << kFineLog) - 1)));
-    const float2 hi = __ldg(tw + (1u << (logn - kFineLog)) + (m >> kFineLog));
+    const float2 hi = __ldg(tw + tw_root(1 << (logn - kFineLog)) + (m >> kFineLog));
     float2 w = cmul(lo, hi);
     if (dir > 0) w.y = -w.y;
     return w;

@@ -113,7 +113,7 @@ __device__ __forceinline__ void tc_tile(const float2 *buf, int sbase, int b0, in
     for (int rr = 0; rr < 2; ++rr) {
         const int b = b0 + g + 8 * rr;
         const int k = b & (Ns - 1);
-        const float2 *twp = tw + (Ns << 4);
+        const float2 *twp = tw + tw_root(Ns << 4);
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             float2 v = buf[sbase + pidx<0, 1>(b + ms[c] * T)];
@@ -389,10 +389,10 @@ __device__ __forceinline__ void tc5_stages(float2 (&v)[16], float2 *xbuf, int j,
         constexpr int LNS = O::LNS;
         if constexpr (LNS > 0) {
             const int k = j & ((1 << LNS) - 1);
-            const float2 *twk = tw + ((1 << LNS) << 4);
+            const float2 *twk = tw + tw_stage16(16 << LNS) + k;
 #pragma unroll
             for (int r = 1; r < 16; ++r) {
-                float2 w = __ldg(twk + r * k);
+                float2 w = __ldg(twk + (r << LNS));
                 if (DIR > 0) w.y = -w.y;
                 v[r] = cmul(v[r], w);
             }

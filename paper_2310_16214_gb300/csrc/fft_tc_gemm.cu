@@ -147,7 +147,7 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t *r) {
 // W_m^e = exp(DIR 2 pi i e / m) from the table of exp(-2 pi i e / m)
 template <int DIR>
 __device__ __forceinline__ float2 root(const float2 *__restrict__ tw, int m, int e) {
-    float2 w = __ldg(tw + m + e);
+    float2 w = __ldg(tw + tw_root(m) + e);
     if (DIR > 0) w.y = -w.y;
     return w;
 }

@@ -146,7 +146,7 @@ constexpr int kBluesteinMaxLog = 23;
 int fft_bluestein_launch(const bplg_plan *plan_m, const void *in, void *out, int64_t n, int64_t batch, int dir,
                          cudaStream_t s);
 
-// twiddle table of the current device (float2 W_M^k at [M + k], M = 2..2^14)
+// twiddle table of the current device (layout: tw_root, tw_stage16 in fft_common.cuh; M = 2..2^14)
 int twiddles_for_current_device(const void **tw);
 
 }  // namespace bplg

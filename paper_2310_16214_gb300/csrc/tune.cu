@@ -300,6 +300,7 @@ struct ModelOp {
     double bpe = 0;     // algorithmic HBM bytes per element
     double acc = 0;     // warp-wide global access instructions per thread
     double lines = 1;   // 128-byte lines per such access
+    double lsu = 0;     // further 128-byte wavefronts of a warp in the load/store unit (exchanges, twiddles)
     bool piped = false; // bulk-copy ring in front of the loads
     bool persistent = false;  // one block per SM looping over tiles, the next tile's loads in flight
     double fp64 = 0;    // FP64 pipe operations per element
@@ -365,19 +366,34 @@ ModelOp model_op(const bplg_plan &p, int64_t n) {
             // products (write A, barrier, issue, commit, mbarrier wait,
             // tensor-memory read: two hand-offs, about 1 us a stage, 32
             // barriers' worth); io 1 gathers fragments
-            m.bars = 2.0 * (K - 1) + (p.op == BPLG_OP_FFT_TC ? (p.io == 0 ? 32.0 : 2.0) * K : 0.0);
+            m.bars = (p.smem_layout == 1 ? 4.0 : 2.0) * (K - 1) +
+                     (p.op == BPLG_OP_FFT_TC ? (p.io == 0 ? 32.0 : 2.0) * K : 0.0);
+            // each exchange moves 8 bytes a lane out and in (two wavefronts each
+            // way, half as much again as four 4-byte passes; unpadded ones conflict), each later stage loads r - 1
+            // twiddles: k fastest in the radix-16 stage blocks, r k apart else
+            m.lsu = (p.smem_layout == 1 ? 6.0 : 4.0) * (K - 1) * r * (p.smem_pad ? 1.0 : 2.0);
+            for (int st = 1, ns = 1 << (logn - (K - 1) * lr); st < K; ++st, ns <<= lr)
+                for (int q = 1; q < r; ++q)
+                    m.lsu += std::max(1.0, std::ceil(std::min(ns, 32) * 8.0 * (spec && r == 16 ? 1 : q) / 128.0));
             if (p.io == 1) {
                 m.instr += r * 4;
                 m.bars += 2;
                 m.acc = 2.0 * std::max(1, r / 2);
                 m.lines = 4;
+                m.lsu += 8.0 * r;  // the staging copies in and out
             } else if (p.io == 0) {
                 m.acc = 2.0 * r;
                 m.lines = std::max(2.0, grouped_lines(tps, 8.0));
             } else {
                 m.acc = 2.0 * std::max(1, r / 2);
                 m.lines = 4;
+                m.bars += 2;  // the tile's arrival and its refill
                 m.piped = true;
+                if (tps < 32) {  // staged through the exchange buffer as io 1
+                    m.instr += r * 4;
+                    m.bars += 2;
+                    m.lsu += 8.0 * r;
+                }
             }
             break;
         }
@@ -452,7 +468,7 @@ double model_kernel(const ModelOp &m, const DevModel &dm, int64_t elems, int64_t
         t_lat,                                                            // latency, b_a blocks (tiles) in flight
         static_cast<double>(elems) * m.bpe / dm.bw,                       // HBM bandwidth
         per_sm_blocks * wpb * m.instr / (kModelIpc * dm.clk),             // issue
-        per_sm_blocks * wpb * m.acc * m.lines * kModelLine / dm.clk,      // lines through the load/store unit
+        per_sm_blocks * wpb * (m.acc * m.lines + m.lsu) * kModelLine / dm.clk,  // load/store unit
         (m.persistent ? 1.0 : per_sm_blocks) * kModelBlockLaunch,         // block launches
         static_cast<double>(elems) * m.fp64 / (sms * kModelFp64PerClk * dm.clk)};  // FP64 pipe
     double s = 0.0;
