@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(MAXT)
         float2 v[16];
 #pragma unroll
         for (int m = 0; m < 16; ++m) v[m] = slot[s * N + j + m * S::T];
-        fft_fixed_stages<16, LOGN, DIR, 0, 0>(v, slot + s * STRIDE, nullptr, j, tw, out + (sig0 + s) * N, active);
+        fft_fixed_stages<16, LOGN, DIR, 0>(v, slot + s * STRIDE, nullptr, j, tw, out + (sig0 + s) * N, active);
         __syncthreads();  // every read of the slot is done: refill it
         const int64_t next = tile + static_cast<int64_t>(NS) * gridDim.x;
         if (tid == 0 && next < ntiles) {
@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(MAXT)
             fence_proxy_async();
             issue(next, q);
         }
-        fft_fixed_stages<16, LOGN, DIR, 1, 0>(v, nullptr, xbuf, j, tw, out + (sig0 + s) * N, active);
+        fft_fixed_stages<16, LOGN, DIR, 1>(v, nullptr, xbuf, j, tw, out + (sig0 + s) * N, active);
     }
 }
 

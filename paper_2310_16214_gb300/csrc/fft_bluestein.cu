@@ -19,8 +19,8 @@
 // For 32 <= M <= 8192 (and no caller plan) the whole chain is one kernel,
 // one signal per M/16 threads: the chirp product is formed as the signal is
 // loaded, the forward M-point transform (the compile-time radix-16 stage
-// schedule) writes its output times G into the shared-memory exchange
-// buffer, the inverse transform reads it back and its last stage writes
+// schedule) leaves its output in registers, where G multiplies it, and the
+// inverse transform starts from there; its last stage writes
 // h_k c_k for k < n straight to global memory.  HBM then carries 16 bytes
 // per element, as for a power-of-two length.  Otherwise (or with a plan for
 // the M-point transforms) the chain runs as three elementwise kernels and
@@ -41,6 +41,17 @@ namespace {
 constexpr int kFusedMinLog = 5, kFusedMaxLog = 13;  // at most 512 threads: 128 registers each
 
 // The fused chain for M = 2^LOGM (radix 16, padded interleaved exchange).
+// Two facts shorten it.  n <= M / 2, so the upper half of the padded input
+// (registers 8 .. 15 of the first stage) is zero and the upper half of the
+// result is not wanted.  And the forward transform's last stage leaves A_k,
+// k = j + r T, in register r of thread j, which is where the inverse's first
+// stage reads it: G multiplies in registers and nothing is exchanged between
+// the transforms.  The kernel is bound by the L1 data pipe (per warp and 512
+// points of M, 259 shared wavefronts in four exchanges and 150 for twiddles,
+// chirp and G) and the issue slots together; with the middle exchange and the
+// full halves it took 0.158 ms at n = 1001, 2^24 points, now 0.133; 0.280 ->
+// 0.232 at n = 4095.  Registers: 128, two blocks per SM at M = 2048; capped at
+// 80 or 64 for more blocks it spills (0.160, 0.184 ms).
 template <int LOGM>
 __global__ void __launch_bounds__(512)
     bluestein_fused_kernel(const float2 *__restrict__ x, float2 *__restrict__ X, const float2 *__restrict__ h,
@@ -59,22 +70,21 @@ __global__ void __launch_bounds__(512)
     const float2 *xs = x + sig * n;
     float2 v[16];
 #pragma unroll
-    for (int m = 0; m < 16; ++m) {
+    for (int m = 0; m < 8; ++m) {
         const int e = j + m * S::T;
         v[m] = active && e < n ? cmul(__ldcs(xs + e), __ldg(h + e)) : make_float2(0.f, 0.f);
     }
-    // forward transform; its output times G goes to the exchange buffer
-    auto to_smem = [&](int pos, float2 val) { buf2[pad_g<16>(pos)] = cmul(val, __ldg(G + pos)); };
-    fft_fixed_stages_st<16, LOGM, -1, 0, 0, true>(v, buf2, buf1, j, tw, to_smem);
-    __syncthreads();
+    // forward transform; output j + r T stays in register r, which is also
+    // where the inverse transform reads its input j + r T
+    fft_fixed_stages_reg<16, LOGM, -1, 0, 0, true>(v, buf2, buf1, j, tw);
 #pragma unroll
-    for (int m = 0; m < 16; ++m) v[m] = buf2[pad_g<16>(j + m * S::T)];
+    for (int r = 0; r < 16; ++r) v[r] = cmul(v[r], __ldg(G + j + r * S::T));
     // inverse transform; X_k = h_k c_k for k < n
     float2 *Xs = X + sig * n;
     auto to_out = [&](int pos, float2 val) {
         if (active && pos < n) __stcs(Xs + pos, cmul(val, __ldg(h + pos)));
     };
-    fft_fixed_stages_st<16, LOGM, 1, 0, 0, true>(v, buf2, buf1, j, tw, to_out);
+    fft_fixed_stages_st<16, LOGM, 1, 0, false, 8>(v, buf2, buf1, j, tw, to_out);
 }
 
 const void *fused_func(int logm) {

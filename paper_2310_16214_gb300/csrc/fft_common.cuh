@@ -104,11 +104,26 @@ __device__ __forceinline__ void dif_layers(float2 (&v)[R]) {
     }
 }
 
-// In-register R-point DFT, natural order in and out.
-template <int R, int DIR>
+// The first layer when v[H .. 2 H - 1] are zero: (a, 0) -> (a, a W_{2H}^k).
+template <int R, int DIR, int K>
+__device__ __forceinline__ void dif_half_layer(float2 (&v)[R]) {
+    if constexpr (K < R / 2) {
+        v[K + R / 2] = cmul_root<DIR, K, R>(v[K]);
+        dif_half_layer<R, DIR, K + 1>(v);
+    }
+}
+
+// In-register R-point DFT, natural order in and out.  HALF: the upper half
+// of the inputs is zero (and v[R / 2 ..] is not read).
+template <int R, int DIR, bool HALF = false>
 __device__ __forceinline__ void dft_codelet(float2 (&v)[R]) {
     if constexpr (R > 1) {
-        dif_layers<R, DIR, R / 2>(v);
+        if constexpr (HALF) {
+            dif_half_layer<R, DIR, 0>(v);
+            dif_layers<R, DIR, R / 4>(v);
+        } else {
+            dif_layers<R, DIR, R / 2>(v);
+        }
         float2 t[R];
 #pragma unroll
         for (int i = 0; i < R; ++i) t[i] = v[bitrev(i, clog2(R))];
@@ -119,15 +134,16 @@ __device__ __forceinline__ void dft_codelet(float2 (&v)[R]) {
 
 // First stage with the lower radix R0 (Ns = 1, no twiddles): the thread's R
 // registers hold R/R0 butterflies, butterfly q using registers q, q+Q, ...
-template <int R, int R0, int DIR>
+// (HALF: registers R/2 .. R-1 are zero, the upper half of every butterfly).
+template <int R, int R0, int DIR, bool HALF = false>
 __device__ __forceinline__ void first_stage_mixed(float2 (&v)[R]) {
     constexpr int Q = R / R0;
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         float2 u[R0];
 #pragma unroll
-        for (int r = 0; r < R0; ++r) u[r] = v[q + r * Q];
-        dft_codelet<R0, DIR>(u);
+        for (int r = 0; r < (HALF ? R0 / 2 : R0); ++r) u[r] = v[q + r * Q];
+        dft_codelet<R0, DIR, HALF>(u);
 #pragma unroll
         for (int r = 0; r < R0; ++r) v[q + r * Q] = u[r];
     }
@@ -203,17 +219,20 @@ struct StageOut {
     }
 };
 
-// The last stage hands each output, with its natural-order position, to
-// store(position, value); with SYNC_LAST the block synchronises first (for a
-// store into the exchange buffer that other threads may still be reading).
-template <int R, int LOGN, int DIR, int LAYOUT, int ST, bool SYNC_LAST = false, class Store>
-__device__ __forceinline__ void fft_fixed_stages_st(float2 (&v)[R], float2 *buf2, float *buf1, int j,
-                                                    const float2 *__restrict__ tw, Store &store) {
+// The stages ST .. last, the last one's outputs left in v: register r of
+// thread j holds position StageOut<last>::base(j) + off(r), which is
+// j + r T whenever the schedule has two stages or more.  HALF_IN: the upper
+// half of the inputs, elements n / 2 .. n - 1 (registers R / 2 .. R - 1), is
+// known to be zero.
+template <int R, int LOGN, int DIR, int LAYOUT, int ST, bool HALF_IN = false>
+__device__ __forceinline__ void fft_fixed_stages_reg(float2 (&v)[R], float2 *buf2, float *buf1, int j,
+                                                     const float2 *__restrict__ tw) {
     using S = FftShape<R, LOGN>;
     using O = StageOut<R, LOGN, ST>;
     constexpr int G = LAYOUT == 0 ? 16 : 32;
+    constexpr bool kHalf = HALF_IN && ST == 0;
     if constexpr (O::kMixed) {
-        first_stage_mixed<R, (1 << S::LR0), DIR>(v);
+        first_stage_mixed<R, (1 << S::LR0), DIR, kHalf>(v);
     } else {
         constexpr int LNS = O::LNS;
         if constexpr (LNS > 0) {
@@ -227,15 +246,10 @@ __device__ __forceinline__ void fft_fixed_stages_st(float2 (&v)[R], float2 *buf2
                 v[r] = cmul(v[r], w);
             }
         }
-        dft_codelet<R, DIR>(v);
+        dft_codelet<R, DIR, kHalf>(v);
     }
-    const int ob = O::base(j);
-    if constexpr (ST == S::NST - 1) {
-        if constexpr (SYNC_LAST) __syncthreads();
-#pragma unroll
-        for (int r = 0; r < R; ++r) store(ob + O::off(r), v[r]);
-    } else {
-        const int pb = pad_g<G>(ob);
+    if constexpr (ST < S::NST - 1) {
+        const int pb = pad_g<G>(O::base(j));
         const int pj = pad_g<G>(j);
         if constexpr (LAYOUT == 0) {
             __syncthreads();
@@ -258,19 +272,34 @@ __device__ __forceinline__ void fft_fixed_stages_st(float2 (&v)[R], float2 *buf2
 #pragma unroll
             for (int m = 0; m < R; ++m) v[m].y = buf1[pj + m * S::T + (m * S::T) / G];
         }
-        fft_fixed_stages_st<R, LOGN, DIR, LAYOUT, ST + 1, SYNC_LAST>(v, buf2, buf1, j, tw, store);
+        fft_fixed_stages_reg<R, LOGN, DIR, LAYOUT, ST + 1, HALF_IN>(v, buf2, buf1, j, tw);
     }
+}
+
+// All stages, then each output handed with its natural-order position to
+// store(position, value); with SYNC_LAST the block synchronises first (for a
+// store into the exchange buffer that other threads may still be reading).
+// Only registers r < OUT are handed over.
+template <int R, int LOGN, int DIR, int LAYOUT, bool SYNC_LAST = false, int OUT = R, class Store>
+__device__ __forceinline__ void fft_fixed_stages_st(float2 (&v)[R], float2 *buf2, float *buf1, int j,
+                                                    const float2 *__restrict__ tw, Store &store) {
+    using O = StageOut<R, LOGN, FftShape<R, LOGN>::NST - 1>;
+    fft_fixed_stages_reg<R, LOGN, DIR, LAYOUT, 0>(v, buf2, buf1, j, tw);
+    const int ob = O::base(j);
+    if constexpr (SYNC_LAST) __syncthreads();
+#pragma unroll
+    for (int r = 0; r < OUT; ++r) store(ob + O::off(r), v[r]);
 }
 
 // The stage schedule with the last stage stored straight to global memory
 // (natural order, streaming stores) when `active`.
-template <int R, int LOGN, int DIR, int LAYOUT, int ST>
+template <int R, int LOGN, int DIR, int LAYOUT>
 __device__ __forceinline__ void fft_fixed_stages(float2 (&v)[R], float2 *buf2, float *buf1, int j,
                                                  const float2 *__restrict__ tw, float2 *gout, bool active) {
     auto store = [&](int pos, float2 val) {
         if (active) __stcs(gout + pos, val);
     };
-    fft_fixed_stages_st<R, LOGN, DIR, LAYOUT, ST>(v, buf2, buf1, j, tw, store);
+    fft_fixed_stages_st<R, LOGN, DIR, LAYOUT>(v, buf2, buf1, j, tw, store);
 }
 
 }  // namespace bplg

@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(MAXT)
     float2 v[R];
 #pragma unroll
     for (int m = 0; m < R; ++m) v[m] = active ? __ldcs(g + m * S::T) : make_float2(0.f, 0.f);
-    fft_fixed_stages<R, LOGN, DIR, LAYOUT, 0>(v, buf2, buf1, j, tw, out + sig * (int64_t(1) << LOGN), active);
+    fft_fixed_stages<R, LOGN, DIR, LAYOUT>(v, buf2, buf1, j, tw, out + sig * (int64_t(1) << LOGN), active);
 }
 
 // Blocks of up to 512 threads get 128 registers per thread (the radix-16

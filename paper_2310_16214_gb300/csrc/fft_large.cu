@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(1024)
         const float2 w = twiddle_n(tw, fine, logn, static_cast<uint32_t>(k1) * static_cast<uint32_t>(n2), DIR);
         __stcs(yo + static_cast<int64_t>(k1) * N2, cmul(val, w));
     };
-    fft_fixed_stages_st<16, LOGN1, DIR, 0, 0>(v, cols + c * col_stride(1 << LOGN1), nullptr, j, tw, store);
+    fft_fixed_stages_st<16, LOGN1, DIR, 0>(v, cols + c * col_stride(1 << LOGN1), nullptr, j, tw, store);
 }
 
 template <int LOGN2, int DIR>
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(1024)
     for (int m = 0; m < 16; ++m) v[m] = __ldcs(g + m * S::T);
     float2 *row = rows + rr * RS;
     auto store = [&](int k2, float2 val) { row[pad_g<16>(k2)] = val; };
-    fft_fixed_stages_st<16, LOGN2, DIR, 0, 0, true>(v, row, nullptr, j, tw, store);
+    fft_fixed_stages_st<16, LOGN2, DIR, 0, true>(v, row, nullptr, j, tw, store);
     __syncthreads();
     // transposed write-out: R consecutive k1 per output column k2
     float2 *o = out + sig * N + k1_0;

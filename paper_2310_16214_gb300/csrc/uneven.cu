@@ -150,7 +150,7 @@ __device__ __noinline__ void fft_unit_fixed(const ItemDesc *items, const UnitDes
     float2 v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = active ? __ldcs(in + m * S::T) : make_float2(0.f, 0.f);
-    fft_fixed_stages<16, LOGN, DIR, 0, 0>(v, b2, nullptr, j, tw, out, active);
+    fft_fixed_stages<16, LOGN, DIR, 0>(v, b2, nullptr, j, tw, out, active);
 }
 
 template <int DIR>
