@@ -183,7 +183,7 @@ int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64
  *          (and no plan) runs a mixed-radix Stockham kernel compiled for
  *          that length: stages of radix 2, 3, 4, 5, 6, 8, 9, 10, 12, 15 or
  *          16, the block's signals in shared memory, the stage twiddles
- *          from a per-n table W_n^e made on the first call with that n
+ *          from a per-n table made on the first call with that n
  *          (float64 on the host, rounded to float32, uploaded
  *          synchronously).
  *          Any other length that is not a power of two runs Bluestein's

@@ -17,9 +17,9 @@ static_assert(kMixedMaxN == kMixedMaxLen, "one limit for the mixed-radix lengths
 namespace {
 
 std::mutex g_mu;
-std::map<std::pair<int, int64_t>, float2 *> g_tables;  // (device, n) -> exp(-2 pi i e / n), e < n
+std::map<std::pair<int, int64_t>, float2 *> g_tables;  // (device, n) -> the stage twiddles (stage_table)
 
-int table_for(int64_t n, const float2 **out) {
+int table_for(int64_t n, const MixedLaunch &ml, const float2 **out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
@@ -29,15 +29,22 @@ int table_for(int64_t n, const float2 **out) {
         *out = it->second;
         return BPLG_OK;
     }
-    std::vector<float2> h(static_cast<size_t>(n));
-    for (int64_t k = 0; k < n; ++k) {
-        const double ang = -2.0 * M_PI * static_cast<double>(k) / static_cast<double>(n);
-        h[static_cast<size_t>(k)] = make_float2(static_cast<float>(std::cos(ang)), static_cast<float>(std::sin(ang)));
+    std::vector<float2> h;
+    h.reserve(static_cast<size_t>(n));
+    int64_t L = ml.radices[0];
+    for (int s = 1; s < ml.stages; L *= ml.radices[s++]) {
+        const int64_t m = n / (L * ml.radices[s]);
+        for (int p = 1; p < ml.radices[s]; ++p)
+            for (int64_t j = 0; j < L; ++j) {
+                const double ang = -2.0 * M_PI * static_cast<double>(p * j * m) / static_cast<double>(n);
+                h.push_back(make_float2(static_cast<float>(std::cos(ang)), static_cast<float>(std::sin(ang))));
+            }
     }
+    if (h.empty()) h.push_back(make_float2(1.f, 0.f));  // one stage: no twiddles
     float2 *d = nullptr;
-    if ((e = cudaMalloc(&d, static_cast<size_t>(n) * sizeof(float2))) != cudaSuccess)
+    if ((e = cudaMalloc(&d, h.size() * sizeof(float2))) != cudaSuccess)
         return cuda_error(e, "mixed-radix twiddles");
-    if ((e = cudaMemcpy(d, h.data(), static_cast<size_t>(n) * sizeof(float2), cudaMemcpyHostToDevice)) !=
+    if ((e = cudaMemcpy(d, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice)) !=
         cudaSuccess) {
         cudaFree(d);
         return cuda_error(e, "mixed-radix twiddles upload");
@@ -68,7 +75,7 @@ int fft_mixed_launch(const void *in, void *out, int64_t n, int64_t batch, int di
         return set_error(BPLG_ERR_UNSUPPORTED_SIZE, "fft (mixed radix): n must be 2^a 3^b 5^c, not a power of two, "
                                                     "at most " + std::to_string(kMixedMaxN));
     const float2 *tw = nullptr;
-    int rc = table_for(n, &tw);
+    int rc = table_for(n, ml, &tw);
     if (rc != BPLG_OK) return rc;
     rc = ensure_smem_attr(ml.fn, ml.smem);
     if (rc != BPLG_OK) return rc;
