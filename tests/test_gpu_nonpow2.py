@@ -103,6 +103,20 @@ def test_tridiag_cr_plan_needs_power_of_two(bp):
         run_tri(bp, sysm, bp.make_plan(bp.OP_TRIDIAG, 128, 2, 1, cr_switch=32, shuffle=1))
 
 
+# Rows that start 1, 2 and 3 elements past a 16-byte boundary, at lengths
+# whose last thread, warp or block is nearly empty or exactly full, and at the
+# longest odd lengths (no room for the shift at n = 32767); in place too.
+@pytest.mark.parametrize("n", [18, 65, 257, 1021, 1022, 1023, 2047, 2049, 8190, 16385, 32766, 32767])
+def test_scan_rows_off_alignment(bp, n):
+    batch = 6
+    x = si.scan_i32(batch, n, stream=900 + n)
+    ref = oracle.scan_i32(x)
+    assert np.array_equal(run_scan(bp, x), ref)
+    buf = to_dev(x.reshape(-1))
+    bp.scan_batched(buf, buf, n, batch)
+    assert np.array_equal(buf.cpu().numpy().reshape(batch, n), ref)
+
+
 # ------------------------------------------------------------------- FFT ----
 
 def tol(n):
