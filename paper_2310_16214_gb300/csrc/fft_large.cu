@@ -24,9 +24,14 @@
 // y lives in a scratch buffer owned by the library (allocated on first use
 // per device and stream, grown to the largest n x batch seen), so in may
 // equal out.
-// W_n^m for n up to 2^24 is a product of two float64-generated tables:
-// W_n^(m mod 4096) (one 4096-entry table per n, cached per device) and
-// W_(n/4096)^(m div 4096) from the main twiddle table.
+// Thread j of a column holds the outputs k1 = j + r T, T = N1 / 16, r < 16, so
+//     W_n^(k1 n2) = W_n^(j n2) W_(16 N2)^(r n2),
+// a product of two float64-generated, once-rounded factors: W_n^m, m < n / 16
+// (a table per n), one load for a thread's 16 outputs; and the stage table
+// [r][n2] of 16 N2 entries (one per N2 and device), read with the column n2
+// across the lanes.  (W_n^(k1 n2 mod 4096) W_n^(4096 (k1 n2 div 4096)) took
+// every output two loads whose lanes lay k1 entries apart, three quarters of
+// the column kernel's L1 work: 0.139 -> 0.127 ms at 2^20 points, 16 signals.)
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -45,16 +50,6 @@ namespace {
 
 constexpr int kLargeMinPassLog = 6;   // each inner transform has 2^6 .. 2^14 points
 constexpr int kLargeMaxPassLog = 14;
-constexpr int kFineLog = 12;          // fine twiddle table: W_n^j, j < 4096
-
-__device__ __forceinline__ float2 twiddle_n(const float2 *__restrict__ tw, const float2 *__restrict__ fine, int logn,
-                                            uint32_t m, int dir) {
-    const float2 lo = __ldg(fine + (m & ((1u << kFineLog) - 1)));
-    const float2 hi = __ldg(tw + tw_root(1 << (logn - kFineLog)) + (m >> kFineLog));
-    float2 w = cmul(lo, hi);
-    if (dir > 0) w.y = -w.y;
-    return w;
-}
 
 __host__ __device__ constexpr int col_stride(int n1) { return n1 + n1 / 16 + 1; }  // float2, skewed
 // rows of the row kernel: a pad of 16 / R float2 (R = rows per block <= 16)
@@ -66,8 +61,8 @@ __host__ __device__ constexpr int row_stride(int n2, int log_rows) {
 
 template <int LOGN1, int DIR>
 __global__ void __launch_bounds__(1024)
-    fft_col_kernel(const float2 *in, float2 *y, const float2 *__restrict__ tw, const float2 *__restrict__ fine,
-                   int logn, int log_cols) {
+    fft_col_kernel(const float2 *in, float2 *y, const float2 *__restrict__ tw, const float2 *__restrict__ root,
+                   const float2 *__restrict__ stage, int logn, int log_cols) {
     using S = FftShape<16, LOGN1>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *cols = reinterpret_cast<float2 *>(smem_raw);
@@ -84,12 +79,20 @@ __global__ void __launch_bounds__(1024)
     float2 v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = __ldcs(g + static_cast<int64_t>(j + m * S::T) * N2);
-    float2 *yo = y + sig * N + n2;
-    auto store = [&](int k1, float2 val) {
-        const float2 w = twiddle_n(tw, fine, logn, static_cast<uint32_t>(k1) * static_cast<uint32_t>(n2), DIR);
-        __stcs(yo + static_cast<int64_t>(k1) * N2, cmul(val, w));
-    };
-    fft_fixed_stages_st<16, LOGN1, DIR, 0>(v, cols + c * col_stride(1 << LOGN1), nullptr, j, tw, store);
+    fft_fixed_stages_reg<16, LOGN1, DIR, 0, 0>(v, cols + c * col_stride(1 << LOGN1), nullptr, j, tw);
+    float2 *yo = y + sig * N + static_cast<int64_t>(j) * N2 + n2;  // output k1 = j + r T
+    float2 base = __ldg(root + j * n2);
+    if (DIR > 0) base.y = -base.y;
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        float2 w = base;
+        if (r > 0) {
+            float2 u = __ldg(stage + r * N2 + n2);
+            if (DIR > 0) u.y = -u.y;
+            w = cmul(base, u);
+        }
+        __stcs(yo + static_cast<int64_t>(r * S::T) * N2, cmul(v[r], w));
+    }
 }
 
 template <int LOGN2, int DIR>
@@ -159,48 +162,65 @@ const void *row_func(int l2) {
     }
 }
 
-// fine twiddles W_n^j (j < 4096) in float64, rounded once
-__global__ void fine_twiddle_kernel(float2 *t, int logn) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= (1 << kFineLog)) return;
+// t[m] = W_n^m, m < count, in float64, rounded once
+__global__ void large_root_kernel(float2 *t, int logn, int64_t count) {
+    const int64_t m = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (m >= count) return;
     double sn, cs;
-    sincospi(-2.0 * static_cast<double>(j) / static_cast<double>(int64_t(1) << logn), &sn, &cs);
-    t[j] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
+    sincospi(-2.0 * static_cast<double>(m) / static_cast<double>(int64_t(1) << logn), &sn, &cs);
+    t[m] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
+}
+
+// t[16 N2 + r N2 + n2] = W_(16 N2)^(r n2) for every N2 of a row pass
+__global__ void large_stage_kernel(float2 *t, int64_t count) {
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= count || i < (int64_t(16) << kLargeMinPassLog)) return;
+    const int logm = 63 - __clzll(static_cast<unsigned long long>(i));  // 16 N2 = 2^logm
+    const int64_t e = i - (int64_t(1) << logm), n2 = int64_t(1) << (logm - 4);
+    double sn, cs;
+    sincospi(-2.0 * static_cast<double>((e / n2) * (e % n2)) / static_cast<double>(int64_t(1) << logm), &sn, &cs);
+    t[i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
 }
 
 std::mutex g_mu;
-std::map<std::pair<int, int>, float2 *> g_fine;       // (device, log n)
+std::map<std::pair<int, int>, float2 *> g_root;  // (device, log n) -> W_n^m; (device, 0) -> the stage tables
 // (device, stream, tag) -> (buffer, bytes)
 std::map<std::tuple<int, cudaStream_t, int>, std::pair<void *, size_t>> g_scratch;
 
-int fine_twiddles(int logn, const float2 **out) {
+// the table of W_n^m, m < n / 16, or (logn 0) the stage tables
+int large_table(int logn, const float2 **out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
     std::lock_guard<std::mutex> lock(g_mu);
-    auto it = g_fine.find({dev, logn});
-    if (it != g_fine.end()) {
+    auto it = g_root.find({dev, logn});
+    if (it != g_root.end()) {
         *out = it->second;
         return BPLG_OK;
     }
+    const int64_t count = logn > 0 ? int64_t(1) << (logn - 4) : int64_t(32) << kLargeMaxPassLog;
     float2 *p = nullptr;
-    e = cudaMalloc(&p, sizeof(float2) << kFineLog);
-    if (e != cudaSuccess) return cuda_error(e, "fine twiddle cudaMalloc");
+    e = cudaMalloc(&p, sizeof(float2) * static_cast<size_t>(count));
+    if (e != cudaSuccess) return cuda_error(e, "large twiddle cudaMalloc");
     cudaStream_t st;
     e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         cudaFree(p);
-        return cuda_error(e, "fine twiddle stream");
+        return cuda_error(e, "large twiddle stream");
     }
-    fine_twiddle_kernel<<<(1 << kFineLog) / 256, 256, 0, st>>>(p, logn);
+    const unsigned blocks = static_cast<unsigned>((count + 255) / 256);
+    if (logn > 0)
+        large_root_kernel<<<blocks, 256, 0, st>>>(p, logn, count);
+    else
+        large_stage_kernel<<<blocks, 256, 0, st>>>(p, count);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaStreamDestroy(st);
     if (e != cudaSuccess) {
         cudaFree(p);
-        return cuda_error(e, "fine twiddle generation");
+        return cuda_error(e, "large twiddle generation");
     }
-    g_fine[{dev, logn}] = p;
+    g_root[{dev, logn}] = p;
     *out = p;
     return BPLG_OK;
 }
@@ -325,9 +345,11 @@ int fft_large_launch(const bplg_plan &p, const void *in, void *out, int64_t n, i
     rc = twiddles_for_current_device(&tw);
     if (rc != BPLG_OK) return rc;
     int logn = ilog2(n);
-    const float2 *fine = nullptr;
-    rc = fine_twiddles(logn, &fine);
+    const float2 *root = nullptr, *stage = nullptr;
+    rc = large_table(logn, &root);
+    if (rc == BPLG_OK) rc = large_table(0, &stage);
     if (rc != BPLG_OK) return rc;
+    stage += n >> (p.n1_log - 4);  // the block of 16 N2
     void *y = nullptr;
     rc = stream_scratch(kScratchLargeFft, static_cast<size_t>(n) * static_cast<size_t>(batch) * sizeof(float2), s, &y);
     if (rc != BPLG_OK) return rc;
@@ -338,7 +360,7 @@ int fft_large_launch(const bplg_plan &p, const void *in, void *out, int64_t n, i
     const float2 *x = static_cast<const float2 *>(in);
     float2 *yy = static_cast<float2 *>(y);
     float2 *o = static_cast<float2 *>(out);
-    void *a0[] = {(void *)&x, (void *)&yy, (void *)&tw, (void *)&fine, &logn, &log_cols};
+    void *a0[] = {(void *)&x, (void *)&yy, (void *)&tw, (void *)&root, (void *)&stage, &logn, &log_cols};
     cudaError_t e = cudaLaunchKernel(l0.func, dim3(static_cast<unsigned>(l0.blocks)), dim3(l0.threads), a0,
                                      static_cast<size_t>(l0.smem), s);
     if (e != cudaSuccess) return launch_error(e, "fft column kernel", l0.func, l0.blocks, l0.threads, l0.smem);

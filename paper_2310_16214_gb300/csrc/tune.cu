@@ -525,12 +525,15 @@ double model_plan_time(const bplg_plan &p, int64_t n, int64_t batch, int regs, i
             return model_kernel(m, dm, n * batch, batch * cnt, threads, rg, sm, static_cast<int>(per_block * len));
         };
         // columns: loads and stores in segments of spb values; rows: loads
-        // whole rows, stores transposed in segments of row_spb values
+        // whole rows, stores transposed in segments of row_spb values, which
+        // cost HBM nothing from 32 bytes on (L2 puts the neighbouring tiles'
+        // segments together; with the columns' cost per segment the model chose
+        // 512-thread blocks at 2^18: 0.132 ms against 0.113)
         const double c = pass(n1, p.spb, n2 / std::max(1, p.spb), regs, smem, grouped_lines(p.spb, 8.0),
                               seg_cost(8.0 * p.spb));
         const double r = pass(n2, p.row_spb, n1 / std::max(1, p.row_spb), regs2 > 0 ? regs2 : regs,
-                              smem2 > 0 ? smem2 : smem, grouped_lines(p.row_spb, 8.0),
-                              0.5 * (1.0 + seg_cost(8.0 * p.row_spb)));
+                              smem2 > 0 ? smem2 : smem, 0.5 * (2.0 + grouped_lines(p.row_spb, 8.0)),
+                              0.5 * (1.0 + std::max(1.0, 32.0 / (8.0 * p.row_spb))));
         return c + r;
     }
     const ModelOp m = model_op(p, n);
