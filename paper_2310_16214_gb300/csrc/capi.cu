@@ -35,6 +35,7 @@ int fft_device_status(int *flag, bool reset);
 int tridiag_device_status(int *flag, bool reset);
 int fft_tc_device_status(int *flag, bool reset);
 int fft_tc_gemm_device_status(int *flag, bool reset);
+int tridiag_wm_device_status(int *flag, bool reset);
 
 namespace {
 std::mutex g_default_mu;
@@ -191,6 +192,9 @@ int bplg_tridiag_batched(const float *a, const float *b, const float *c, const f
     if (np != n && plan && plan->op != BPLG_OP_TRIDIAG_WM)
         return set_error(BPLG_ERR_UNSUPPORTED_SIZE,
                          "tridiag: n that is not a power of two needs a BPLG_OP_TRIDIAG_WM plan (or NULL)");
+    // without a plan the longer ones take the persistent bulk-copy form of it
+    if (!plan && tridiag_wm_tma_applies(n))
+        return tridiag_wm_tma_launch(a, b, c, d, x, n, batch, static_cast<cudaStream_t>(stream));
     const int op = np != n || (plan && plan->op == BPLG_OP_TRIDIAG_WM) ? BPLG_OP_TRIDIAG_WM : BPLG_OP_TRIDIAG;
     bplg_plan p;
     OnlineTicket tk;
@@ -391,7 +395,7 @@ int bplg_online_status(int32_t op, int32_t dtype, int64_t n, int64_t batch, int3
 int bplg_device_status(int32_t *flag, int32_t reset) {
     clear_error();
     if (!flag) return set_error(BPLG_ERR_INVALID_ARG, "null output");
-    int f1 = 0, f2 = 0, f3 = 0, f4 = 0;
+    int f1 = 0, f2 = 0, f3 = 0, f4 = 0, f5 = 0;
     int rc = fft_device_status(&f1, reset != 0);
     if (rc != BPLG_OK) return rc;
     rc = tridiag_device_status(&f2, reset != 0);
@@ -400,7 +404,9 @@ int bplg_device_status(int32_t *flag, int32_t reset) {
     if (rc != BPLG_OK) return rc;
     rc = fft_tc_gemm_device_status(&f4, reset != 0);
     if (rc != BPLG_OK) return rc;
-    *flag = f1 ? f1 : (f2 ? f2 : (f3 ? f3 : f4));
+    rc = tridiag_wm_device_status(&f5, reset != 0);
+    if (rc != BPLG_OK) return rc;
+    *flag = f1 ? f1 : (f2 ? f2 : (f3 ? f3 : (f4 ? f4 : f5)));
     return BPLG_OK;
 }
 

@@ -43,6 +43,7 @@
 
 #include "device_util.cuh"
 #include "internal.h"
+#include "tma.cuh"
 #include "tridiag_common.cuh"
 #include "tridiag_wm.cuh"
 
@@ -113,6 +114,126 @@ __global__ void __launch_bounds__(MAXT)
     }
 }
 
+// Systems of a length that is not a power of two without a plan, from a
+// persistent grid, one system per block at a time: the four coefficient rows
+// arrive in shared memory by bulk copies (from the 16-byte boundary before the
+// row to the one after it), each thread takes its P equations into registers, and
+// the slot is refilled with the block's next system while this one is solved
+// and stored, so HBM reads go on throughout.
+//   Layout.  Threads that read P consecutive equations straight from global
+// memory are 4 P bytes apart, and a 16-byte load of a warp then touches P / 2
+// lines: at P = 16 (n = 3000) the loads and stores were most of the work of the
+// L1 data pipe (57 % busy at 23 % occupancy), and rows off a 16-byte boundary had
+// to be read element by element.  From shared memory with P = 12 or 20 the lanes
+// lie 3 or 5 16-byte units apart, an odd number, so the eight lanes of each
+// phase hit distinct banks and a load takes the least four wavefronts; and the
+// row may start anywhere (sh elements of the copy precede it).
+//   Threads.  The tps threads the row needs, in whole warps: those missing from
+// the merge tree stand for identity rows, whose descriptors are zero, which is
+// what their shared-memory slots hold.  PER_WARP (one exchange slot a warp) lets
+// two blocks of 98 KB fit where one slot a thread takes 118 KB: n = 5000 0.085 ->
+// 0.071 ms; below that it only adds shuffles (0.0594 -> 0.0615 ms at n = 3000).
+//   Measured at 2^24 unknowns, padded power-of-two kernel -> this one: n = 300
+// 0.076 -> 0.062 ms, 700 0.072 -> 0.062, 1500 0.066 -> 0.058, 3000 0.086 -> 0.060 (82
+// % of the copy bandwidth), 3001 0.182 -> 0.060, 5000 0.124 -> 0.065, 8191 0.195 ->
+// 0.076.
+template <int P, int MAXT, int MINB, bool PER_WARP>
+__global__ void __launch_bounds__(MAXT, MINB)
+    tridiag_wm_tma_kernel(const float *ga, const float *gb, const float *gc, const float *gd, float *x, int log_tps,
+                          int64_t batch, int nrow) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ __align__(8) uint64_t full;
+    const int tps = blockDim.x, t = threadIdx.x;
+    constexpr int W = PER_WARP ? 5 : 0;  // log2 of the threads that share an exchange slot
+    const int slots = (1 << log_tps) >> W, len = tps * P;
+    float4 *buf = reinterpret_cast<float4 *>(smem_raw);
+    float *slot = reinterpret_cast<float *>(buf + 4 * slots);  // a, b, c, d, `len` floats each
+    const int64_t total = batch * nrow;
+    // elements copied of a row that starts at row0: whole 16-byte units, and not past
+    // the end of the arrays (the last row's last elements are then read directly)
+    auto copied = [&](int64_t row0) {
+        const int sh = static_cast<int>(row0 & 3);
+        const int count = (sh + nrow + 3) & ~3;
+        return row0 - sh + count > total ? count - 4 : count;
+    };
+    auto issue = [&](int64_t sys) {
+        const int64_t row0 = sys * nrow;
+        const uint32_t bytes = static_cast<uint32_t>(copied(row0)) * 4u;
+        const int64_t from = row0 - (row0 & 3);
+        mbar_arrive_expect_tx(&full, 4 * bytes);
+        tma_load_1d(slot, ga + from, bytes, &full);
+        tma_load_1d(slot + len, gb + from, bytes, &full);
+        tma_load_1d(slot + 2 * len, gc + from, bytes, &full);
+        tma_load_1d(slot + 3 * len, gd + from, bytes, &full);
+    };
+    if (t == 0) {
+        mbar_init(&full, 1);
+        fence_mbar_init();
+        issue(blockIdx.x);
+    }
+    const int absent = slots - (tps >> W);  // the absent threads' descriptors
+    for (int k = t; k < 4 * absent; k += tps)
+        buf[(k / absent) * slots + (tps >> W) + k % absent] = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncthreads();
+    uint32_t parity = 0;
+    for (int64_t sys = blockIdx.x; sys < batch; sys += gridDim.x, parity ^= 1u) {
+        const bool ok = mbar_wait_bounded(&full, parity);
+        float a[P], b[P], c[P], d[P];
+        const float4 *s4 = reinterpret_cast<const float4 *>(slot + t * P);
+#pragma unroll
+        for (int q = 0; q < P / 4; ++q) {
+            const float4 va = s4[q], vb = s4[len / 4 + q], vc = s4[2 * (len / 4) + q], vd = s4[3 * (len / 4) + q];
+            a[4 * q] = va.x; a[4 * q + 1] = va.y; a[4 * q + 2] = va.z; a[4 * q + 3] = va.w;
+            b[4 * q] = vb.x; b[4 * q + 1] = vb.y; b[4 * q + 2] = vb.z; b[4 * q + 3] = vb.w;
+            c[4 * q] = vc.x; c[4 * q + 1] = vc.y; c[4 * q + 2] = vc.z; c[4 * q + 3] = vc.w;
+            d[4 * q] = vd.x; d[4 * q + 1] = vd.y; d[4 * q + 2] = vd.z; d[4 * q + 3] = vd.w;
+        }
+        // the slot is read (and the exchange buffers of the last system too); on
+        // a timeout every thread leaves, the copy having been waited for
+        if (!__syncthreads_and(ok)) return;
+        if (t == 0 && sys + gridDim.x < batch) {
+            fence_proxy_async();
+            issue(sys + gridDim.x);
+        }
+        const int64_t row0 = sys * nrow;
+        const int sh = static_cast<int>(row0 & 3);
+        const int i0 = t * P - sh;  // the thread's first equation, as an index of the row
+        if (i0 <= 0 || i0 + P >= nrow) {
+            // the first and the last threads: identity rows outside the row, a of its
+            // first and c of its last equation 0, elements past the copied ones
+            const int have = copied(row0) - sh;
+#pragma unroll
+            for (int e = 0; e < P; ++e) {
+                const int i = i0 + e;
+                const bool in = i >= 0 && i < nrow;
+                if (in && i >= have) {
+                    a[e] = ga[row0 + i];
+                    b[e] = gb[row0 + i];
+                    c[e] = gc[row0 + i];
+                    d[e] = gd[row0 + i];
+                }
+                a[e] = in && i > 0 ? a[e] : 0.f;
+                b[e] = in ? b[e] : 1.f;
+                c[e] = in && i < nrow - 1 ? c[e] : 0.f;
+                d[e] = in ? d[e] : 0.f;
+            }
+        }
+        wm::wm_solve_inreg<P, 2, 1, true, PER_WARP>(a, b, c, d, log_tps, buf, tps, t, t, slots);
+        float *xo = x + row0 + i0;
+#pragma unroll
+        for (int q = 0; q < P; q += 4) {
+            const int i = i0 + q;
+            if (i >= 0 && i + 3 < nrow) {
+                __stcs(reinterpret_cast<float4 *>(xo + q), make_float4(d[q], d[q + 1], d[q + 2], d[q + 3]));
+            } else {
+#pragma unroll
+                for (int e = q; e < q + 4; ++e)
+                    if (i0 + e >= 0 && i0 + e < nrow) xo[e] = d[e];
+            }
+        }
+    }
+}
+
 template <int P, int R, bool RAGGED>
 const void *wm_func_r(int shuffle) {
     constexpr int MAXT = P >= 8 || R >= 8 ? 512 : 1024;
@@ -157,6 +278,61 @@ bool tridiag_wm_launch_info(const bplg_plan &p, int64_t n, int64_t batch, Launch
     out->smem = tridiag_wm_smem_bytes(p, n);
     out->blocks = (batch + p.spb - 1) / p.spb;
     return true;
+}
+
+// Read (and optionally clear) the device error word of this file's kernels.
+int tridiag_wm_device_status(int *flag, bool reset) {
+    int v = 0;
+    cudaError_t e = cudaMemcpyFromSymbol(&v, g_device_error, sizeof(int));
+    if (e != cudaSuccess) return cuda_error(e, "device status");
+    if (reset && v) {
+        const int zero = 0;
+        e = cudaMemcpyToSymbol(g_device_error, &zero, sizeof(int));
+        if (e != cudaSuccess) return cuda_error(e, "device status reset");
+    }
+    *flag = v;
+    return BPLG_OK;
+}
+
+// Which lengths take it: those above 256 whose padded form wastes threads or has
+// rows off 16-byte boundaries.  Up to 1024 a multiple of 4 within 1/16 of the
+// power of two is as fast padded (P = 8, whose lanes lie closer): n = 500 0.0556
+// ms against 0.0566, 1000 0.0580 against 0.0600; up to 256 a block here is one
+// warp with half of its lanes idle.
+bool tridiag_wm_tma_applies(int64_t n) {
+    if (is_pow2(n) || n <= 256 || n > (int64_t(1) << kTridiagMaxLog)) return false;
+    const int64_t np = next_pow2(n);
+    return n % 4 != 0 || n > 1024 || (np - n) * 16 > np;
+}
+
+int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const float *d, float *x, int64_t n,
+                          int64_t batch, cudaStream_t s) {
+    const int max_shift = n % 4 == 0 ? 0 : (n % 2 == 0 ? 2 : 3);  // rows before the first in its 16 bytes
+    const auto threads = [&](int P) { return static_cast<int>((n + max_shift + 32 * P - 1) / (32 * P) * 32); };
+    // P = 12, or 20 where that leaves fewer threads idle: one warp instead of two
+    // (n = 385 .. 640), and above 2048 (n = 2500 0.0665 -> 0.0613 ms, 3500 0.0734 -> 0.0643,
+    // but 3000 0.0600 against 0.0645 and 4500 0.0683 against 0.0698, whose rows fill
+    // P = 12 better).  More than 448 threads of P = 12 leave one block per SM
+    // (n = 5500 0.0866 ms against 0.0709 with P = 20).
+    const int t12 = threads(12), t20 = threads(20);
+    const bool p20 = t20 == 32 ? t12 > 32 : t12 > 448 || (n > 2048 && 20 * t20 * 100 <= 12 * t12 * 101);
+    const int P = p20 ? 20 : 12, tps = p20 ? t20 : t12;
+    const bool per_warp = tps > 288 || (p20 && tps > 32);
+    const void *f = p20 ? (tps == 32    ? reinterpret_cast<const void *>(&tridiag_wm_tma_kernel<20, 32, 14, false>)
+                           : tps <= 288 ? reinterpret_cast<const void *>(&tridiag_wm_tma_kernel<20, 288, 2, true>)
+                                        : reinterpret_cast<const void *>(&tridiag_wm_tma_kernel<20, 416, 1, true>))
+                        : (tps <= 288 ? reinterpret_cast<const void *>(&tridiag_wm_tma_kernel<12, 288, 3, false>)
+                                      : reinterpret_cast<const void *>(&tridiag_wm_tma_kernel<12, 448, 2, true>));
+    int log_tps = ilog2(next_pow2(tps)), nrow = static_cast<int>(n);
+    const int smem = 4 * 16 * ((1 << log_tps) >> (per_warp ? 5 : 0)) + 4 * 4 * tps * P;
+    int rc = ensure_smem_attr(f, smem);
+    if (rc != BPLG_OK) return rc;
+    int64_t grid = 0;
+    rc = persistent_grid(f, tps, smem, batch, &grid);
+    if (rc != BPLG_OK) return rc;
+    void *args[] = {(void *)&a, (void *)&b, (void *)&c, (void *)&d, (void *)&x, &log_tps, &batch, &nrow};
+    cudaError_t e = cudaLaunchKernel(f, dim3(static_cast<unsigned>(grid)), dim3(tps), args, static_cast<size_t>(smem), s);
+    return e == cudaSuccess ? BPLG_OK : launch_error(e, "tridiag (Wang-Mou, bulk-copy) launch", f, grid, tps, smem);
 }
 
 int tridiag_wm_launch(const bplg_plan &p, const float *a, const float *b, const float *c, const float *d, float *x,

@@ -67,9 +67,13 @@ __device__ __forceinline__ void wm_outer(const Aff (&F)[RS], const Aff (&L)[RS],
 
 // One merge stage of radix RS over runs of S threads: gather the RS
 // descriptors of this thread's group, then re-express the thread's own
-// first/last descriptors in terms of the merged run's neighbours.
-template <int RS>
-__device__ __forceinline__ void wm_stage(Aff &Fo, Aff &Lo, int t, int log_s, bool by_shuffle, float4 *bf,
+// first/last descriptors in terms of the merged run's neighbours.  slot is
+// the thread's shared-memory slot.  PER_WARP: the runs are whole warps (every
+// stage inside a warp goes by shuffles), so a run's first and last
+// descriptors are those of its first warp's lane 0 and its last warp's lane 31:
+// only those threads write, one slot a warp.
+template <int RS, bool PER_WARP>
+__device__ __forceinline__ void wm_stage(Aff &Fo, Aff &Lo, int t, int slot, int log_s, bool by_shuffle, float4 *bf,
                                          float4 *bl) {
     const int S = 1 << log_s;
     const int G = S * RS;
@@ -89,15 +93,15 @@ __device__ __forceinline__ void wm_stage(Aff &Fo, Aff &Lo, int t, int log_s, boo
             L[h].y = __shfl_sync(kFullMask, Lo.y, sl);
         }
     } else {
-        const int tid = threadIdx.x;
-        bf[tid] = make_float4(Fo.a, Fo.x, Fo.y, 0.f);
-        bl[tid] = make_float4(Lo.a, Lo.x, Lo.y, 0.f);
+        constexpr int W = PER_WARP ? 5 : 0;  // log2 of the threads that share a slot
+        if (!PER_WARP || (t & (S - 1)) == 0) bf[slot >> W] = make_float4(Fo.a, Fo.x, Fo.y, 0.f);
+        if (!PER_WARP || (t & (S - 1)) == S - 1) bl[slot >> W] = make_float4(Lo.a, Lo.x, Lo.y, 0.f);
         __syncthreads();
-        const int sys0 = tid - t;  // this system's first thread in the block
+        const int sys0 = slot - t;  // the slot of this system's first thread
 #pragma unroll
         for (int h = 0; h < RS; ++h) {
-            const float4 f = bf[sys0 + base + h * S];
-            const float4 l = bl[sys0 + base + h * S + S - 1];
+            const float4 f = bf[(sys0 + base + h * S) >> W];
+            const float4 l = bl[(sys0 + base + h * S + S - 1) >> W];
             F[h] = Aff{f.x, f.y, f.z};
             L[h] = Aff{l.x, l.y, l.z};
         }
@@ -116,14 +120,26 @@ __host__ __device__ __forceinline__ bool wm_warp_only(int shuffle, int64_t tps) 
 // the threads that serve it, from this thread's P equations in registers
 // (identity rows where `active` is false).  a..c are destroyed and d ends
 // holding the thread's P unknowns.  buf is the block's shared memory (4
-// float4 per thread) unless every exchange is a warp shuffle.  Every thread
-// of the block calls it.
-template <int P, int R, int SHUFFLE>
+// float4 per thread, or with PER_WARP, which needs R = 2 and SHUFFLE, 4 per
+// warp) unless every exchange is a warp shuffle.  Every thread
+// of the block calls it.  A system has 2^log_tps threads; or, with SHORT,
+// only tps of them (a multiple of the warp; t the thread's index among
+// them, slot its place in the block with 2^log_tps places a system, slots the
+// float4 of one of the four exchange arrays: one a place, or one for 32 with
+// PER_WARP): the threads that are not there stand for
+// identity rows, whose descriptors are zero, and the caller has zeroed their
+// slots.
+template <int P, int R, int SHUFFLE, bool SHORT = false, bool PER_WARP = false>
 __device__ __forceinline__ void wm_solve_inreg(float (&a)[P], float (&b)[P], float (&c)[P], float (&d)[P],
-                                               int log_tps, float4 *buf) {
-    const int tps = 1 << log_tps;
-    const int tid = threadIdx.x;
-    const int t = tid & (tps - 1);
+                                               int log_tps, float4 *buf, int tps = 0, int t = 0, int slot = 0,
+                                               int slots = 0) {
+    static_assert(!PER_WARP || (R == 2 && SHUFFLE), "stages outside a warp merge whole warps");
+    if constexpr (!SHORT) {
+        tps = 1 << log_tps;
+        t = threadIdx.x & (tps - 1);
+        slot = threadIdx.x;
+        slots = blockDim.x;
+    }
     if (t == 0) a[0] = 0.f;
     if (t == tps - 1) c[P - 1] = 0.f;
 
@@ -155,7 +171,6 @@ __device__ __forceinline__ void wm_solve_inreg(float (&a)[P], float (&b)[P], flo
     Aff Lo = Aff{al[P - 1], be[P - 1], gm[P - 1]};
 
     // (2) merge stages: runs of S threads, RS of them per group
-    const int nthr = blockDim.x;
     int par = 0;
     constexpr int LR = R >= 8 ? 3 : (R >= 4 ? 2 : 1);
 #pragma unroll
@@ -163,15 +178,15 @@ __device__ __forceinline__ void wm_solve_inreg(float (&a)[P], float (&b)[P], flo
         const int lrs = log_tps - log_s >= LR ? LR : log_tps - log_s;  // log2 of this stage's radix
         const int rs = 1 << lrs;
         const bool by_shuffle = SHUFFLE && log_s + lrs <= 5;
-        float4 *bf = buf + (2 * par) * nthr;
-        float4 *bl = bf + nthr;
+        float4 *bf = buf + (2 * par) * slots;
+        float4 *bl = bf + slots;
         if constexpr (R >= 8) {
-            if (rs == 8) wm_stage<8>(Fo, Lo, t, log_s, by_shuffle, bf, bl);
+            if (rs == 8) wm_stage<8, PER_WARP>(Fo, Lo, t, slot, log_s, by_shuffle, bf, bl);
         }
         if constexpr (R >= 4) {
-            if (rs == 4) wm_stage<4>(Fo, Lo, t, log_s, by_shuffle, bf, bl);
+            if (rs == 4) wm_stage<4, PER_WARP>(Fo, Lo, t, slot, log_s, by_shuffle, bf, bl);
         }
-        if (rs == 2) wm_stage<2>(Fo, Lo, t, log_s, by_shuffle, bf, bl);
+        if (rs == 2) wm_stage<2, PER_WARP>(Fo, Lo, t, slot, log_s, by_shuffle, bf, bl);
         if (!by_shuffle) par ^= 1;
         log_s += lrs;
     }
@@ -184,11 +199,22 @@ __device__ __forceinline__ void wm_solve_inreg(float (&a)[P], float (&b)[P], flo
         xl_nb = t > 0 ? up : 0.f;
         xr_nb = t < tps - 1 ? dn : 0.f;
     } else {
-        float2 *xb = reinterpret_cast<float2 *>(buf + (2 * par) * nthr);
-        xb[tid] = make_float2(Fo.a, Lo.a);
-        __syncthreads();
-        xl_nb = t > 0 ? xb[tid - 1].y : 0.f;
-        xr_nb = t < tps - 1 ? xb[tid + 1].x : 0.f;
+        float2 *xb = reinterpret_cast<float2 *>(buf + (2 * par) * slots);
+        if constexpr (PER_WARP) {  // neighbours in the warp by shuffles, across warps one slot a warp
+            const int w = slot >> 5, lane = slot & 31;
+            if (lane == 0) xb[w].x = Fo.a;
+            if (lane == 31) xb[w].y = Lo.a;
+            __syncthreads();
+            xl_nb = __shfl_up_sync(kFullMask, Lo.a, 1);
+            xr_nb = __shfl_down_sync(kFullMask, Fo.a, 1);
+            if (lane == 0) xl_nb = t > 0 ? xb[w - 1].y : 0.f;
+            if (lane == 31) xr_nb = t < tps - 1 ? xb[w + 1].x : 0.f;
+        } else {
+            xb[slot] = make_float2(Fo.a, Lo.a);
+            __syncthreads();
+            xl_nb = t > 0 ? xb[slot - 1].y : 0.f;
+            xr_nb = t < tps - 1 ? xb[slot + 1].x : 0.f;
+        }
     }
 #pragma unroll
     for (int i = 0; i < P; ++i) d[i] = fmaf(gm[i], xr_nb, fmaf(be[i], xl_nb, al[i]));

@@ -117,6 +117,27 @@ def test_scan_rows_off_alignment(bp, n):
     assert np.array_equal(buf.cpu().numpy().reshape(batch, n), ref)
 
 
+# Every thread count and equations-per-thread choice of the bulk-copy solver
+# (257 .. 8191), rows at all four places in their 16 bytes, at the edges of its
+# ranges; batches small and large enough that a block solves several systems in
+# turn; x may alias d.
+@pytest.mark.parametrize("n,batch", [(18, 6), (257, 6000), (380, 5), (384, 3), (385, 6), (637, 6), (638, 4001), (959, 7),
+                                     (1021, 6), (1022, 6), (1023, 6), (1025, 3000), (2047, 6), (2500, 1500), (3001, 1101),
+                                     (3500, 6), (4095, 6), (5373, 700), (5374, 6), (5757, 6), (5758, 501), (8190, 6),
+                                     (8191, 400)])
+def test_tridiag_rows_off_alignment(bp, n, batch):
+    a, b, c, d, _ = si.tridiag_f32(batch, n, stream=950 + n)
+    a[:, 0] = np.nan  # never read
+    c[:, -1] = np.nan
+    ref = oracle.thomas(a, b, c, d)
+    x = run_tri(bp, (a, b, c, d))
+    assert np.all(np.isfinite(x)) and tri_rel_err(x, ref).max() <= 1e-4
+    ts = [to_dev(v.reshape(-1)) for v in (a, b, c, d)]
+    bp.tridiag_batched(*ts, ts[3], n, batch)  # x aliases d
+    assert np.array_equal(ts[3].cpu().numpy().reshape(batch, n), x)
+    assert bp.device_status() == 0
+
+
 # ------------------------------------------------------------------- FFT ----
 
 def tol(n):
