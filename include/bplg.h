@@ -160,10 +160,10 @@ typedef struct {
  *   dtype  BPLG_I32 (two's-complement wrap-around, bit-exact) or BPLG_F32.
  *   in,out device, [batch][n] of dtype; in == out (in place) is allowed.
  *   n      1 <= n <= 32768; batch >= 1.  A power of two runs its own plan;
- *          any other n runs the plan of the next power of two n' (plan->n ==
- *          n', or plan NULL), the rows read as if padded with zeros to n'
- *          (element-wise accesses; rows stay n apart, nothing past n is
- *          written).
+ *          any other n runs a plan of the next power of two n' (plan->n ==
+ *          n'; plan NULL: the tuned plan of n' if there is one, else one
+ *          chosen for n itself), the rows read as if padded with zeros to n'
+ *          (rows stay n apart, nothing outside a row is read or written).
  * Errors: INVALID_ARG, UNSUPPORTED_SIZE, INVALID_PLAN, CUDA. */
 int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64_t batch,
                       const bplg_plan *plan, void *stream);

@@ -117,11 +117,15 @@ int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64
     if (n < 1 || batch < 1) return set_error(BPLG_ERR_INVALID_ARG, "scan: n and batch must be >= 1");
     if (n > (int64_t(1) << kScanMaxLog)) return set_error(BPLG_ERR_UNSUPPORTED_SIZE, "scan: n must be <= 32768");
     if (!aligned16(in) || !aligned16(out)) return set_error(BPLG_ERR_INVALID_ARG, "scan: buffers must be 16-byte aligned");
-    // any other n runs the plan of the next power of two, padded with zeros
+    // any other n runs a plan of the next power of two n', padded with zeros
     const int64_t np = next_pow2(n);
     bplg_plan p;
     OnlineTicket tk;
-    int rc = resolve_plan(BPLG_OP_SCAN, dtype, np, batch, plan, &p, np == n ? &tk : nullptr);
+    int rc = BPLG_OK;
+    if (np == n || plan)
+        rc = resolve_plan(BPLG_OP_SCAN, dtype, np, batch, plan, &p, np == n ? &tk : nullptr);
+    else if (!cache_lookup(BPLG_OP_SCAN, dtype, np, batch, &p))  // a tuned plan of n', else the ragged rule's
+        p = scan_ragged_plan(n);
     if (rc != BPLG_OK) return rc;
     p.n = static_cast<int32_t>(np);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
