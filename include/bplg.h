@@ -275,11 +275,10 @@ int bplg_fft_batched_noalloc(const void *in, void *out, int64_t n, int64_t batch
  *           n' (a BPLG_OP_TRIDIAG_WM plan with plan->n == n', or NULL): the
  *           system is padded with identity rows (a = c = 0, b = 1, d = 0),
  *           c[s][n-1] is taken as 0, rows stay n apart and nothing past n is
- *           written.  Without a plan most such n above 256 run a persistent
- *           form of the solver with its own tiling (whatever plan is cached
- *           for n'), fed by bulk copies in whole 16-byte units: up to three
- *           elements on either side of a row may be read, none outside the
- *           arrays.
+ *           written.  With plan NULL and no tuned plan of n' most such n
+ *           above 256 run a persistent form of the solver with its own tiling,
+ *           fed by bulk copies in whole 16-byte units: up to three elements on
+ *           either side of a row may be read, none outside the arrays.
  * No pivoting: the systems must be safe for elimination without pivoting
  * (e.g. strictly diagonally dominant).  Pivots are inverted with the fast
  * float32 reciprocal (__fdividef(1, x)), which gives 0 for |x| > 2^126, so

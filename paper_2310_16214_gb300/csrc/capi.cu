@@ -196,11 +196,12 @@ int bplg_tridiag_batched(const float *a, const float *b, const float *c, const f
     if (np != n && plan && plan->op != BPLG_OP_TRIDIAG_WM)
         return set_error(BPLG_ERR_UNSUPPORTED_SIZE,
                          "tridiag: n that is not a power of two needs a BPLG_OP_TRIDIAG_WM plan (or NULL)");
-    // without a plan the longer ones take the persistent bulk-copy form of it
-    if (!plan && tridiag_wm_tma_applies(n))
+    // without a plan (given or tuned for n') the longer ones take the persistent
+    // bulk-copy form of it
+    bplg_plan p;
+    if (!plan && tridiag_wm_tma_applies(n) && !cache_lookup(BPLG_OP_TRIDIAG_WM, BPLG_F32, np, batch, &p))
         return tridiag_wm_tma_launch(a, b, c, d, x, n, batch, static_cast<cudaStream_t>(stream));
     const int op = np != n || (plan && plan->op == BPLG_OP_TRIDIAG_WM) ? BPLG_OP_TRIDIAG_WM : BPLG_OP_TRIDIAG;
-    bplg_plan p;
     OnlineTicket tk;
     int rc = resolve_plan(op, BPLG_F32, np, batch, plan, &p, np == n ? &tk : nullptr);
     if (rc != BPLG_OK) return rc;

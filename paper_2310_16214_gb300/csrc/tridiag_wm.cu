@@ -325,7 +325,8 @@ int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const 
                                       : reinterpret_cast<const void *>(&tridiag_wm_tma_kernel<12, 448, 2, true>));
     int log_tps = ilog2(next_pow2(tps)), nrow = static_cast<int>(n);
     const int smem = 4 * 16 * ((1 << log_tps) >> (per_warp ? 5 : 0)) + 4 * 4 * tps * P;
-    int rc = ensure_smem_attr(f, smem);
+    int rc = check_grid(batch, "tridiag (Wang-Mou)");  // one block a system at most, as the padded kernel
+    if (rc == BPLG_OK) rc = ensure_smem_attr(f, smem);
     if (rc != BPLG_OK) return rc;
     int64_t grid = 0;
     rc = persistent_grid(f, tps, smem, batch, &grid);
