@@ -161,12 +161,31 @@ def _ptr(x) -> Optional[int]:
     return x.data_ptr()
 
 
+_torch = None       # the torch module once a call has needed it
+_raw_stream = None  # device index -> current cudaStream_t, where this torch has it
+
+
+def _current_stream() -> Optional[int]:
+    """torch's current stream on the current device, None without CUDA.
+
+    Read as the raw handle where torch offers that: building the Stream object
+    that torch.cuda.current_stream() returns took 3 of the 9 us of a small call.
+    """
+    global _torch, _raw_stream
+    if _torch is None:
+        import torch
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _torch = torch
+    if _raw_stream is not None and _torch.cuda.is_initialized():
+        return _raw_stream(_torch._C._cuda_getDevice())
+    if _torch.cuda.is_available():
+        return _torch.cuda.current_stream().cuda_stream
+    return None
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        if torch.cuda.is_available():
-            return torch.cuda.current_stream().cuda_stream
-        return None
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
