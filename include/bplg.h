@@ -186,6 +186,9 @@ int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64
  *          from a per-n table made on the first call with that n
  *          (float64 on the host, rounded to float32, uploaded
  *          synchronously).
+ *          Any other length up to 12288 whose prime factors are at most 31
+ *          (and no plan) runs the same stages planned at run time, with prime
+ *          radices 7 to 31, and a table made the same way.
  *          Any other length that is not a power of two runs Bluestein's
  *          chirp identity: X_k = h_k sum_j (x_j h_j) conj(h_{k-j}) with
  *          h_m = exp(dir pi i m^2 / n), a cyclic convolution of length

@@ -147,6 +147,9 @@ int stream_scratch(int tag, size_t bytes, cudaStream_t s, void **out);
 constexpr int64_t kMixedMaxN = 12288;
 bool fft_mixed_supported(int64_t n);
 int fft_mixed_launch(const void *in, void *out, int64_t n, int64_t batch, int dir, cudaStream_t s);
+// prime factors up to 31, not all of them 2, 3 or 5; n <= 12288 (fft_prime.cuh)
+bool fft_prime_applies(int64_t n);
+int fft_prime_launch(const void *in, void *out, int64_t n, int64_t batch, int dir, cudaStream_t s);
 constexpr int kBluesteinMaxLog = 23;
 int fft_bluestein_launch(const bplg_plan *plan_m, const void *in, void *out, int64_t n, int64_t batch, int dir,
                          cudaStream_t s);

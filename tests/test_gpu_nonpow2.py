@@ -167,6 +167,38 @@ def test_fft_bluestein_vs_dft(bp, n):
         assert fft_rel_err(X, ref).max() <= tol(n), (n, direction)
 
 
+# lengths with a prime factor above 31: the fused Bluestein kernel at both ends of
+# its range (M = 128 .. 8192)
+@pytest.mark.parametrize("n", [37, 74, 1009, 2039, 4093])
+def test_fft_bluestein_large_primes_vs_dft(bp, n):
+    batch = 5 if n <= 1009 else 2
+    x = si.fft_c64(batch, n, stream=820 + n)
+    for direction in (-1, 1):
+        assert fft_rel_err(run_fft(bp, x, direction), oracle.dft(x, direction)).max() <= tol(n), (n, direction)
+
+
+# prime radices 7 .. 31: every radix first, in the middle and last, one stage to
+# five, one signal a block and many (the last block not full), the longest
+# length; in place too.  Above 2100 points against numpy's float64 FFT.
+@pytest.mark.parametrize("n,batch", [(7, 700), (11, 5), (13, 3), (17, 250), (19, 4), (23, 4), (29, 4), (31, 70), (34, 61), (77, 31),
+                                     (143, 20), (221, 16), (323, 4), (437, 6), (527, 5), (713, 3), (899, 3), (961, 5),
+                                     (1001, 4), (1547, 3), (2001, 2), (2002, 3), (4004, 3), (4199, 2), (9009, 2),
+                                     (10571, 2), (12012, 2), (12276, 3)])
+def test_fft_prime_radices(bp, n, batch):
+    x = si.fft_c64(batch, n, stream=840 + n)
+    for direction in (-1, 1):
+        X = run_fft(bp, x, direction)
+        if n <= 2100:
+            ref = oracle.dft(x, direction)
+        else:
+            z = x.astype(np.complex128)
+            ref = np.fft.fft(z, axis=1) if direction < 0 else np.fft.ifft(z, axis=1, norm="forward")
+        assert fft_rel_err(X, ref).max() <= tol(n), (n, direction)
+    buf = c64_to_dev(x.reshape(-1))
+    bp.fft_batched(buf, buf, n, batch, -1)
+    assert np.array_equal(c64_from_dev(buf).reshape(batch, n), run_fft(bp, x, -1))
+
+
 # 2^a 3^b 5^c (not a power of two, at most 12288): the mixed-radix Stockham
 # kernels (one per length, radices 2 .. 16); small lengths several signals a
 # block (ragged last block)
