@@ -224,7 +224,8 @@ int bplg_fft_batched(const void *in, void *out, int64_t n, int64_t batch, int32_
  *             exactly, and undoes it at the end).
  *   n        power of two, 512 <= n <= 16384; in, out as bplg_fft_batched.
  *   plan     op BPLG_OP_FFT_TC (radix 16; P, spb, io as above), or NULL
- *            (the GB300 cost model's choice).
+ *            (the GB300 cost model's choice; at n = 512, untuned, the io 0
+ *            kernel, which the plan space offers from 1024 points on).
  * Errors: INVALID_ARG, UNSUPPORTED_SIZE, INVALID_PLAN, CUDA. */
 int bplg_fft_tc_batched(const void *in, void *out, int64_t n, int64_t batch, int32_t dir,
                         int32_t precision, const bplg_plan *plan, void *stream);

@@ -174,8 +174,11 @@ int bplg_fft_tc_batched(const void *in, void *out, int64_t n, int64_t batch, int
     if (!aligned16(in) || !aligned16(out)) return set_error(BPLG_ERR_INVALID_ARG, "fft tc: buffers must be 16-byte aligned");
     bplg_plan p;
     OnlineTicket tk;
+    const bool untuned512 = !plan && n == 512 && !cache_lookup(BPLG_OP_FFT_TC, BPLG_F32, n, batch, &p);
     int rc = resolve_plan(BPLG_OP_FFT_TC, BPLG_F32, n, batch, plan, &p, &tk);
     if (rc != BPLG_OK) return rc;
+    if (untuned512 && !tk.applies)
+        return fft_tc512_launch(in, out, batch, dir, precision, static_cast<cudaStream_t>(stream));
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (tk.e0) cudaEventRecord(tk.e0, s);
     rc = fft_tc_launch(p, in, out, n, batch, dir, precision, s);

@@ -49,6 +49,20 @@ def test_every_plan(bp, n, prec):
             assert err <= 1e-5 * math.log2(n), (p, d, prec, err)
 
 
+@pytest.mark.parametrize("batch", [1, 3, 4, 5, 2050])
+def test_default_512_runs_tcgen05(bp, batch):
+    """512 points without a plan: the tcgen05 kernel, four signals a block."""
+    z = si.fft_c64(batch, 512, stream=660 + batch)
+    for d in (-1, 1):
+        ref = oracle.fft(z, d)
+        for prec in (0, 1):
+            assert fft_rel_err(run(bp, z, d, prec), ref).max() <= 1e-5 * 9
+    buf = c64_to_dev(z)
+    bp.fft_tc_batched(buf, buf, 512, batch, -1, precision=1)
+    assert fft_rel_err(c64_from_dev(buf), oracle.fft(z, -1)).max() <= 1e-5 * 9
+    assert bp.device_status() == 0
+
+
 @pytest.mark.parametrize("n", [1024, 4096, 16384])
 def test_precision_configuration_sampled(bp, n):
     # batch = 2^26 / N signals, default plan, both precisions
