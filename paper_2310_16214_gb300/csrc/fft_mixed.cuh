@@ -201,7 +201,42 @@ struct Plan {
     int minb = 0;              // blocks per SM the register budget is set for
     int vmax = 0;              // complex values a thread holds across a barrier
     bool dbl = false;          // two buffers a signal (one barrier a stage instead of two)
+    int pitch[kMaxStages] = {}; // rows of m_s entries that stage s writes, this many places apart
+    int sig = 0, sig2 = 0;     // shared-memory places of a signal in its buffer, in the second one
 };
+
+// Shared-memory wavefronts of 16 lanes (a half-warp of 8-byte accesses hits 16
+// places per wavefront) from lane t0 on, lane t at row t / row, column t % row of
+// an array of rows `pitch` places apart.
+constexpr int half_warp_wavefronts(int t0, int row, int pitch) {
+    int hits[16] = {}, most = 0;
+    for (int t = t0; t < t0 + 16; ++t) {
+        const int c = ++hits[((t / row) * pitch + t % row) % 16];
+        most = c > most ? c : most;
+    }
+    return most;
+}
+
+// Pitch of the rows of m entries between two stages: stage s writes rows of m =
+// r' m' (its lanes run along them), stage s + 1, of radix r', reads runs of m' at
+// the starts of consecutive rows.  Unpadded, the reads of a short m' fall on few
+// banks (rows of 30, runs of 5: three wavefronts for one); the pitch takes the
+// fewest wavefronts of both, of equal ones the smallest, and is m unless that
+// saves a tenth (n = 4000 gained nothing from 3 %).
+constexpr int best_pitch(int m, int m_next) {
+    int best = m, best_cost = 1 << 30, plain = 0;
+    for (int pitch = m; pitch < m + 16 && (pitch == m || 4 * (pitch - m) <= m); ++pitch) {
+        int cost = 0;
+        for (int t0 = 0; t0 < 240; t0 += 16)
+            cost += half_warp_wavefronts(t0, m, pitch) + half_warp_wavefronts(t0, m_next, pitch);
+        if (pitch == m) plain = cost;
+        if (cost < best_cost) {
+            best = pitch;
+            best_cost = cost;
+        }
+    }
+    return 10 * best_cost <= 9 * plain ? best : m;
+}
 
 constexpr int rmin_of(const Plan &p) {
     int m = 1 << 30;
@@ -242,7 +277,7 @@ constexpr void search(int n, int left, int from, Plan &cur, Plan &best) {
     }
 }
 
-constexpr Plan mixed_plan(int n) {
+constexpr Plan mixed_plan_padded(int n, bool pad) {
     Plan cur{}, p{};
     search(n, n, 0, cur, p);
     const int rmin = rmin_of(p), rmax0 = rmax_of(p);
@@ -276,7 +311,19 @@ constexpr Plan mixed_plan(int n) {
     int lower = 2 * p.vmax + 12;
     if (lower < 32) lower = 32;
     if (rmax >= 12 && lower < 48) lower = 48;
-    const int sm1 = p.k > 1 ? n * 8 : 0;
+    int even = 0, odd = 0;  // places the stages s = 0, 2, .. and 1, 3, .. write
+    for (int s = 0, rows = 1; s + 1 < p.k; ++s) {
+        rows *= p.r[s];
+        p.pitch[s] = pad ? best_pitch(n / rows, n / rows / p.r[s + 1]) : n / rows;
+        int &most = s % 2 ? odd : even;
+        most = rows * p.pitch[s] > most ? rows * p.pitch[s] : most;
+    }
+    p.sig = even > odd ? even : odd;
+    if (p.sig * 8 > kSmemPerBlock) {  // no room for the padding
+        p.sig = even = odd = n;
+        for (int s = 0, rows = 1; s + 1 < p.k; ++s) p.pitch[s] = n / (rows *= p.r[s]);
+    }
+    const int sm1 = p.k > 1 ? p.sig * 8 : 0;
     auto blocks_per_sm = [&](int threads, int smem, int regs) {
         int blocks = 2048 / threads;
         const int by_regs = 65536 / (threads * ((regs + 7) / 8 * 8));
@@ -314,8 +361,29 @@ constexpr Plan mixed_plan(int n) {
     }
     auto blocks_at = [&](int smem) { return blocks_per_sm(p.threads, smem, best_regs); };
     // a second buffer when it costs no block per SM
-    p.dbl = p.k > 2 && 2 * p.spb * sm1 <= kSmemPerBlock && blocks_at(2 * p.spb * sm1) >= p.minb;
+    const int sm2 = (even + odd) * 8;
+    p.dbl = p.k > 2 && p.spb * sm2 <= kSmemPerBlock && blocks_at(p.spb * sm2) >= p.minb;
+    if (p.dbl) {
+        p.sig = even;
+        p.sig2 = odd;
+    }
     return p;
+}
+
+// Shared memory of an SM's blocks, with the 1 KB the system keeps of each.
+constexpr int smem_per_sm(const Plan &p) { return p.minb * (p.spb * (p.sig + p.sig2) * 8 + 1024); }
+
+// Padded rows, unless they take an SM's blocks beyond 196 KB: the next size of the
+// shared memory leaves 28 KB of L1 instead of 60, too little for the twiddle table
+// (n = 1500, 3000 and 6000: 0.0535, 0.0615, 0.0663 ms unpadded, 0.064, 0.070, 0.080
+// padded).  Measured at 2^24 points, unpadded -> padded: n = 576 0.0577 -> 0.0502 ms, 1000
+// 0.0561 -> 0.0495, 1536 0.0524 -> 0.0473, 2700 0.0663 -> 0.0533, 5120 0.0741 -> 0.0639, 8000
+// 0.0782 -> 0.0703.
+constexpr Plan mixed_plan(int n) {
+    const Plan padded = mixed_plan_padded(n, true);
+    if (smem_per_sm(padded) <= 196 * 1024) return padded;
+    const Plan plain = mixed_plan_padded(n, false);
+    return smem_per_sm(plain) <= 196 * 1024 ? plain : padded;
 }
 
 constexpr int stage_len_before(const Plan &p, int s) {
@@ -352,7 +420,7 @@ __device__ __forceinline__ void stage_in(const float2 *src, const float2 *__rest
         float2 u[R];
 #pragma unroll
         for (int p = 0; p < R; ++p) {
-            const int e = R * j * m + k + p * m;
+            const int e = (S == 0 ? R * j * m : j * P.pitch[S > 0 ? S - 1 : 0]) + k + p * m;
             if constexpr (S == 0)
                 u[p] = live ? __ldcs(src + e) : make_float2(0.f, 0.f);
             else
@@ -385,11 +453,10 @@ __device__ __forceinline__ void stage_out(float2 *dst, int t, bool act, bool liv
         const int j = b / m, k = b - j * m;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
-            const int e = j * m + k + q * lm;
             if constexpr (LAST) {
-                if (live) __stcs(dst + e, v[i * R + q]);
+                if (live) __stcs(dst + j * m + k + q * lm, v[i * R + q]);
             } else {
-                dst[e] = v[i * R + q];
+                dst[j * P.pitch[S] + k + q * (L * P.pitch[S])] = v[i * R + q];
             }
         }
     }
@@ -427,8 +494,8 @@ __global__ void __launch_bounds__(mixed_plan(N).threads, mixed_plan(N).minb)
     const int t = static_cast<int>(threadIdx.x) - s * P.t;
     const int64_t sig = static_cast<int64_t>(blockIdx.x) * P.spb + s;
     const bool live = act && sig < batch;
-    float2 *buf = reinterpret_cast<float2 *>(smem_raw) + (act ? s : 0) * N;
-    float2 *buf2 = buf + (P.dbl ? P.spb * N : 0);
+    float2 *buf = reinterpret_cast<float2 *>(smem_raw) + (act ? s : 0) * P.sig;
+    float2 *buf2 = P.dbl ? reinterpret_cast<float2 *>(smem_raw) + P.spb * P.sig + (act ? s : 0) * P.sig2 : buf;
     float2 v[P.vmax];
     stage_in<N, 0, DIR>(in + sig * N, tw, t, act, live, v);
     stages_from<N, 1, DIR>(buf, buf2, out + sig * N, tw, t, act, live, v);
@@ -472,7 +539,7 @@ bool fill(int n, int dir, MixedLaunch *o) {
                     : reinterpret_cast<const void *>(&fft_mixed_kernel<N, 1>);
     o->threads = P.threads;
     o->spb = P.spb;
-    o->smem = P.k > 1 ? (P.dbl ? 2 : 1) * P.spb * N * static_cast<int>(sizeof(float2)) : 0;  // one stage: none
+    o->smem = P.k > 1 ? P.spb * (P.sig + P.sig2) * static_cast<int>(sizeof(float2)) : 0;  // one stage: none
     o->stages = P.k;
     for (int i = 0; i < kMaxStages; ++i) o->radices[i] = i < P.k ? P.r[i] : 0;
     return true;
