@@ -223,10 +223,13 @@ struct StageOut {
 // thread j holds position StageOut<last>::base(j) + off(r), which is
 // j + r T whenever the schedule has two stages or more.  HALF_IN: the upper
 // half of the inputs, elements n / 2 .. n - 1 (registers R / 2 .. R - 1), is
-// known to be zero.
-template <int R, int LOGN, int DIR, int LAYOUT, int ST, bool HALF_IN = false>
+// known to be zero.  TURN (layout 0, two stages or more): the last stage is
+// done by other threads than the ones before it: this one reads butterfly
+// last_j of the signal exchanged in last_buf.
+template <int R, int LOGN, int DIR, int LAYOUT, int ST, bool HALF_IN = false, bool TURN = false>
 __device__ __forceinline__ void fft_fixed_stages_reg(float2 (&v)[R], float2 *buf2, float *buf1, int j,
-                                                     const float2 *__restrict__ tw) {
+                                                     const float2 *__restrict__ tw,
+                                                     const float2 *last_buf = nullptr, int last_j = 0) {
     using S = FftShape<R, LOGN>;
     using O = StageOut<R, LOGN, ST>;
     constexpr int G = LAYOUT == 0 ? 16 : 32;
@@ -248,7 +251,18 @@ __device__ __forceinline__ void fft_fixed_stages_reg(float2 (&v)[R], float2 *buf
         }
         dft_codelet<R, DIR, kHalf>(v);
     }
-    if constexpr (ST < S::NST - 1) {
+    if constexpr (TURN && ST == S::NST - 2) {
+        static_assert(LAYOUT == 0, "the turn needs whole complex values in the exchange");
+        const int pb = pad_g<G>(O::base(j));
+        const int pj = pad_g<G>(last_j);
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < R; ++r) buf2[pb + O::off(r) + O::off(r) / G] = v[r];
+        __syncthreads();
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[m] = last_buf[pj + m * S::T + (m * S::T) / G];
+        fft_fixed_stages_reg<R, LOGN, DIR, LAYOUT, ST + 1>(v, nullptr, nullptr, last_j, tw);
+    } else if constexpr (ST < S::NST - 1) {
         const int pb = pad_g<G>(O::base(j));
         const int pj = pad_g<G>(j);
         if constexpr (LAYOUT == 0) {
@@ -272,7 +286,7 @@ __device__ __forceinline__ void fft_fixed_stages_reg(float2 (&v)[R], float2 *buf
 #pragma unroll
             for (int m = 0; m < R; ++m) v[m].y = buf1[pj + m * S::T + (m * S::T) / G];
         }
-        fft_fixed_stages_reg<R, LOGN, DIR, LAYOUT, ST + 1, HALF_IN>(v, buf2, buf1, j, tw);
+        fft_fixed_stages_reg<R, LOGN, DIR, LAYOUT, ST + 1, HALF_IN, TURN>(v, buf2, buf1, j, tw, last_buf, last_j);
     }
 }
 

@@ -18,8 +18,12 @@
 //   banks), and output k1 of column n2 is multiplied by W_n^(k1 n2) and
 //   stored to y[k1][n2], again spb contiguous values per row.
 //   Kernel 2 takes row_spb adjacent rows per block: loads are contiguous
-//   within a row; the outputs are collected in shared memory and written
-//   transposed, X[k1 + N1 k2] for row_spb consecutive k1 at a time.
+//   within a row; the last stage's butterflies are dealt out with the row
+//   fastest across the threads, so their outputs go straight from the
+//   registers to X[k1 + N1 k2], row_spb consecutive k1 at a time.
+//   (Collecting the outputs in shared memory first cost a third exchange, 6.3 M of
+//   its wavefronts where two take 4.2 M, in a kernel bound by them: 2^20 points, 16
+//   signals, both kernels 0.1285 -> 0.1209 ms; 2^16, 256 signals 0.0962 -> 0.0942.)
 //
 // y lives in a scratch buffer owned by the library (allocated on first use
 // per device and stream, grown to the largest n x batch seen), so in may
@@ -53,7 +57,7 @@ constexpr int kLargeMaxPassLog = 14;
 
 __host__ __device__ constexpr int col_stride(int n1) { return n1 + n1 / 16 + 1; }  // float2, skewed
 // rows of the row kernel: a pad of 16 / R float2 (R = rows per block <= 16)
-// puts the R rows of the transposed read-out 32 / R banks apart, so the 16
+// puts the R rows of the last stage's reads 32 / R banks apart, so the 16
 // lanes of each half-warp (16 / R columns x R rows) hit 16 bank pairs
 __host__ __device__ constexpr int row_stride(int n2, int log_rows) {
     return n2 + n2 / 16 + (log_rows <= 4 ? (16 >> log_rows) : 1);
@@ -117,17 +121,14 @@ __global__ void __launch_bounds__(1024)
     float2 v[16];
 #pragma unroll
     for (int m = 0; m < 16; ++m) v[m] = __ldcs(g + m * S::T);
-    float2 *row = rows + rr * RS;
-    auto store = [&](int k2, float2 val) { row[pad_g<16>(k2)] = val; };
-    fft_fixed_stages_st<16, LOGN2, DIR, 0, true>(v, row, nullptr, j, tw, store);
-    __syncthreads();
-    // transposed write-out: R consecutive k1 per output column k2
-    float2 *o = out + sig * N + k1_0;
-    for (int e = tid; e < R * N2; e += blockDim.x) {
-        const int r2 = e & (R - 1);
-        const int k2 = e >> log_rows;
-        __stcs(o + r2 + N1 * k2, rows[r2 * RS + pad_g<16>(k2)]);
-    }
+    // the last stage by thread (j2, r2), r2 fastest: its outputs, k2 = j2 + m T
+    // of row r2, go from the registers to R consecutive k1 per column
+    const int r2 = tid & (R - 1);
+    const int j2 = tid >> log_rows;
+    fft_fixed_stages_reg<16, LOGN2, DIR, 0, 0, false, true>(v, rows + rr * RS, nullptr, j, tw, rows + r2 * RS, j2);
+    float2 *o = out + sig * N + k1_0 + r2 + N1 * j2;
+#pragma unroll
+    for (int m = 0; m < 16; ++m) __stcs(o + m * (N1 * S::T), v[m]);
 }
 
 template <int DIR>

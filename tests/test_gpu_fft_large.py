@@ -48,6 +48,22 @@ def test_every_plan_2_15(bp):
             assert err <= 1e-5 * math.log2(n), (p, d, err)
 
 
+@pytest.mark.parametrize("row_log", range(6, 15))
+def test_every_row_count_per_block(bp, row_log):
+    # the last stage of the row pass is dealt to the threads row fastest: each row
+    # length with every number of rows a block can take, the same bound as above
+    logn = max(15, row_log + 6)
+    n = 1 << logn
+    z = si.fft_c64(2, n, stream=100 + row_log)
+    ref = {d: oracle.fft(z, d) for d in (-1, 1)}
+    plans = {p.row_spb: p for p in bp.enumerate_plans(bp.OP_FFT, bp.F32, n) if p.n1_log == logn - row_log}
+    assert plans
+    for p in plans.values():
+        for d in (-1, 1):
+            assert fft_rel_err(run(bp, z, d, p), ref[d]).max() <= 1e-5 * logn, (p, d)
+    assert bp.device_status() == 0
+
+
 @pytest.mark.parametrize("logn", [16, 18, 20, 22])
 def test_default_plan(bp, logn):
     n = 1 << logn
