@@ -17,13 +17,13 @@
 // from a table per n (stage_table below), computed on the host in float64
 // and rounded to float32, like the power-of-two tables.
 //
-// Radices 16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2: the 3- and 5-point DFTs
+// Radices 25, 24, 20, 18, 16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2: the 3- and 5-point DFTs
 // written out, the composite ones as two factors with their inner twiddles
 // computed at compile time (float64 series, rounded once).  Because n, the
 // radices and every stage's m' are compile-time constants, the index
 // arithmetic folds into constants and immediates, and each kernel holds the
 // code of its own radices only (so its registers are those of its largest
-// codelet).  The plan (mixed_plan below): the fewest stages, radices in
+// codelet).  The plan (kernel_plan below): the fewest stages, radices in
 // non-increasing order; T threads per signal, each doing at most B
 // butterflies a stage (one in the smallest-radix stage unless n / r_min
 // exceeds 1024 threads, or one in the largest-radix stage when the radices
@@ -169,6 +169,14 @@ __device__ __forceinline__ void dft_any(float2 (&v)[R]) {
         dft_two_factor<4, 3, DIR>(v);
     } else if constexpr (R == 15) {
         dft_two_factor<3, 5, DIR>(v);
+    } else if constexpr (R == 18) {
+        dft_two_factor<2, 9, DIR>(v);
+    } else if constexpr (R == 20) {
+        dft_two_factor<4, 5, DIR>(v);
+    } else if constexpr (R == 24) {
+        dft_two_factor<3, 8, DIR>(v);
+    } else if constexpr (R == 25) {
+        dft_two_factor<5, 5, DIR>(v);
     } else {
         dft_codelet<R, DIR>(v);
     }
@@ -176,11 +184,15 @@ __device__ __forceinline__ void dft_any(float2 (&v)[R]) {
 
 // ---------------------------------------------------------------- plan
 
-constexpr int kNumRadices = 11;
-constexpr int kRadices[kNumRadices] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
+constexpr int kNumWide = 4;  // the radices above 16, first in the list (kernel_plan)
+constexpr int kNumRadices = kNumWide + 11;
+constexpr int kRadices[kNumRadices] = {25, 24, 20, 18, 16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
 constexpr int kMaxStages = 8;
 constexpr int kMaxThreads = 1024;
-constexpr int kSmemPerSm = 233472;    // shared memory of one SM available to blocks
+constexpr int kSmemPerSm = 196 * 1024; // shared memory of one SM given to several blocks: beyond it
+                                       // 28 KB of L1 are left instead of 60 (at 2^24 points, 228 KB allowed -> this:
+                                       // n = 768 0.0584 -> 0.0455 ms, 1600 0.0619 -> 0.0463, 1800 0.0599 -> 0.0512,
+                                       // 6561 0.0782 -> 0.0667)
 constexpr int kSmemPerBlock = 232448; // the opt-in limit of one block
 
 constexpr bool is_smooth(int n) {
@@ -277,30 +289,37 @@ constexpr void search(int n, int left, int from, Plan &cur, Plan &best) {
     }
 }
 
-constexpr Plan mixed_plan_padded(int n, bool pad) {
+constexpr Plan plan_of(int n, int from, bool pad) {
     Plan cur{}, p{};
-    search(n, n, 0, cur, p);
+    search(n, n, from, cur, p);
     const int rmin = rmin_of(p), rmax0 = rmax_of(p);
-    if (rmax0 >= 2 * rmin && n / rmax0 <= kMaxThreads) {
+    auto values = [&](int t) {  // most complex values a thread of t holds in a stage
+        int most = 0;
+        for (int s = 0; s < p.k; ++s) {
+            const int v = (n / p.r[s] + t - 1) / t * p.r[s];
+            most = v > most ? v : most;
+        }
+        return most;
+    };
+    if (rmax0 >= 2 * rmin && n / rmax0 <= kMaxThreads && (rmax0 < 18 || 4 * values(n / rmax0) <= 5 * rmax0)) {
         // radices at least a factor two apart: one butterfly a thread in the
         // largest-radix stage and several in the smaller-radix ones, rather
         // than idle threads in the large one (measured faster at n = 375,
-        // 2000 and 3000; slower at 1620 and 6000, whose radices are closer)
+        // 2000 and 3000; slower at 1620 and 6000, whose radices are closer);
+        // above radix 16 only while no stage holds over a quarter more than
+        // the largest radix (n = 3200, 20 x 16 x 10, 32 values 0.0615 ms, one
+        // butterfly a thread 0.0533; 4000, 20 x 20 x 10, 20 values 0.0527 against 0.0619)
         p.t = n / rmax0;
         p.b = (n / rmin + p.t - 1) / p.t;
     } else {
         p.b = bfly_per_thread(n, rmin);
         p.t = (n / rmin + p.b - 1) / p.b;
     }
-    p.vmax = 0;
-    for (int s = 0; s < p.k; ++s) {
-        const int bs = (n / p.r[s] + p.t - 1) / p.t;
-        p.vmax = bs * p.r[s] > p.vmax ? bs * p.r[s] : p.vmax;
-    }
+    p.vmax = values(p.t);
     // Block shape and register budget.  The budget is at least what the
     // values held across a barrier need (two registers each, plus room for
     // indices, addresses and the codelets' temporaries; 48 for the 12- to
-    // 16-point codelets, which need them to keep their loads in flight).
+    // 16-point codelets, which need them to keep their loads in flight; 56 from 18 on).
     // Blocks of at most 256 threads where a signal allows: many small blocks, so that one block's barriers stall few
     // threads and the blocks of an SM drift apart, some loading while others
     // compute.  Among the shapes that keep at least 1280 threads (40 warps)
@@ -311,6 +330,7 @@ constexpr Plan mixed_plan_padded(int n, bool pad) {
     int lower = 2 * p.vmax + 12;
     if (lower < 32) lower = 32;
     if (rmax >= 12 && lower < 48) lower = 48;
+    if (rmax >= 18 && lower < 56) lower = 56;
     int even = 0, odd = 0;  // places the stages s = 0, 2, .. and 1, 3, .. write
     for (int s = 0, rows = 1; s + 1 < p.k; ++s) {
         rows *= p.r[s];
@@ -326,7 +346,12 @@ constexpr Plan mixed_plan_padded(int n, bool pad) {
     const int sm1 = p.k > 1 ? p.sig * 8 : 0;
     auto blocks_per_sm = [&](int threads, int smem, int regs) {
         int blocks = 2048 / threads;
-        const int by_regs = 65536 / (threads * ((regs + 7) / 8 * 8));
+        // From radix 15 on a warp's registers are counted in the quarter of the SM
+        // they lie in: counted whole, the compiler got 40 registers for a budget of 48
+        // and spilled (n = 75 0.0626 -> 0.0556 ms, 240 0.0537 -> 0.0431, 675 0.0731 ->
+        // 0.0534; 2304 0.0474 -> 0.0494).  Below, the 40 do, with more warps.
+        const int by_regs = rmax >= 15 ? 4 * (512 / ((regs + 7) / 8 * 8)) / (threads / 32)
+                                       : 65536 / (threads * ((regs + 7) / 8 * 8));
         if (by_regs < blocks) blocks = by_regs;
         if (smem > 0 && kSmemPerSm / (smem + 1024) < blocks) blocks = kSmemPerSm / (smem + 1024);
         if (blocks > 32) blocks = 32;
@@ -373,17 +398,34 @@ constexpr Plan mixed_plan_padded(int n, bool pad) {
 // Shared memory of an SM's blocks, with the 1 KB the system keeps of each.
 constexpr int smem_per_sm(const Plan &p) { return p.minb * (p.spb * (p.sig + p.sig2) * 8 + 1024); }
 
-// Padded rows, unless they take an SM's blocks beyond 196 KB: the next size of the
-// shared memory leaves 28 KB of L1 instead of 60, too little for the twiddle table
-// (n = 1500, 3000 and 6000: 0.0535, 0.0615, 0.0663 ms unpadded, 0.064, 0.070, 0.080
-// padded).  Measured at 2^24 points, unpadded -> padded: n = 576 0.0577 -> 0.0502 ms, 1000
-// 0.0561 -> 0.0495, 1536 0.0524 -> 0.0473, 2700 0.0663 -> 0.0533, 5120 0.0741 -> 0.0639, 8000
-// 0.0782 -> 0.0703.
-constexpr Plan mixed_plan(int n) {
-    const Plan padded = mixed_plan_padded(n, true);
-    if (smem_per_sm(padded) <= 196 * 1024) return padded;
-    const Plan plain = mixed_plan_padded(n, false);
-    return smem_per_sm(plain) <= 196 * 1024 ? plain : padded;
+// Padded rows, unless they take a block that fills an SM beyond 196 KB (the next
+// size of the shared memory leaves 28 KB of L1 instead of 60, too little for the
+// twiddle table: n = 12150 0.106 ms unpadded, 0.113 padded).
+constexpr Plan padded_plan(int n, int from) {
+    const Plan padded = plan_of(n, from, true);
+    if (smem_per_sm(padded) <= kSmemPerSm) return padded;
+    const Plan plain = plan_of(n, from, false);
+    return smem_per_sm(plain) <= kSmemPerSm ? plain : padded;
+}
+// The plan with radices up to 16.
+constexpr Plan mixed_plan(int n) { return padded_plan(n, kNumWide); }
+
+// The plan of a length's kernel: with radices 25, 24, 20 and 18 too where they save
+// a stage, an exchange of every value through shared memory and its barriers (the
+// L1 data pipe, 80 % busy, bounds these kernels).  Not up to 288 points, where
+// one or two stages of them leave a signal too few threads (n = 24 0.0475 ms with
+// radices 6 and 4, 0.111 with one of 24; 288 0.0485 and 0.0573); not with a stage of
+// a radix below 9 or a second one less than half the first, whose threads idle in the large
+// stage or hold too much in the small ones (1250 0.0576, 0.0627; 2500 0.0593, 0.0658;
+// 3125 0.0699, 0.0997); and not where one block is left to an SM instead of several
+// (9375 0.0825, 0.0848).  Elsewhere, measured at 2^24 points, radices up to 16 ->
+// these: n = 400 0.0595 -> 0.0474 ms, 2000 0.0601 -> 0.0533, 3000 0.0619 -> 0.0557,
+// 5120 0.0660 -> 0.0498, 8640 0.103 -> 0.0612, 12000 0.101 -> 0.0829.
+constexpr Plan kernel_plan(int n) {
+    const Plan narrow = mixed_plan(n), wide = padded_plan(n, 0);
+    const bool take = n > 288 && wide.k < narrow.k && wide.r[wide.k - 1] >= 9 && 2 * wide.r[1] >= wide.r[0] &&
+                      (wide.minb > 1 || narrow.minb == 1);
+    return take ? wide : narrow;
 }
 
 constexpr int stage_len_before(const Plan &p, int s) {
@@ -409,7 +451,7 @@ constexpr int stage_table(const Plan &p, int s) { return stage_len_before(p, s) 
 template <int N, int S, int DIR>
 __device__ __forceinline__ void stage_in(const float2 *src, const float2 *__restrict__ tw, int t, bool act, bool live,
                                          float2 *v) {
-    constexpr Plan P = mixed_plan(N);
+    constexpr Plan P = kernel_plan(N);
     constexpr int R = P.r[S], L = stage_len_before(P, S), m = N / (L * R), nb = N / R;
     constexpr int BS = (nb + P.t - 1) / P.t;
 #pragma unroll
@@ -443,7 +485,7 @@ __device__ __forceinline__ void stage_in(const float2 *src, const float2 *__rest
 // Stage S's outputs to the shared buffer, or (LAST) to global memory
 template <int N, int S, bool LAST>
 __device__ __forceinline__ void stage_out(float2 *dst, int t, bool act, bool live, const float2 *v) {
-    constexpr Plan P = mixed_plan(N);
+    constexpr Plan P = kernel_plan(N);
     constexpr int R = P.r[S], L = stage_len_before(P, S), m = N / (L * R), nb = N / R, lm = L * m;
     constexpr int BS = (nb + P.t - 1) / P.t;
 #pragma unroll
@@ -470,7 +512,7 @@ __device__ __forceinline__ void stage_out(float2 *dst, int t, bool act, bool liv
 template <int N, int S, int DIR>
 __device__ __forceinline__ void stages_from(float2 *buf, float2 *buf2, float2 *gout, const float2 *__restrict__ tw,
                                             int t, bool act, bool live, float2 *v) {
-    constexpr Plan P = mixed_plan(N);
+    constexpr Plan P = kernel_plan(N);
     if constexpr (S == P.k) {
         stage_out<N, S - 1, true>(gout, t, act, live, v);
     } else {
@@ -484,10 +526,10 @@ __device__ __forceinline__ void stages_from(float2 *buf, float2 *buf2, float2 *g
 }
 
 template <int N, int DIR>
-__global__ void __launch_bounds__(mixed_plan(N).threads, mixed_plan(N).minb)
+__global__ void __launch_bounds__(kernel_plan(N).threads, kernel_plan(N).minb)
     fft_mixed_kernel(const float2 *__restrict__ in, float2 *__restrict__ out, const float2 *__restrict__ tw,
                      int64_t batch) {
-    constexpr Plan P = mixed_plan(N);
+    constexpr Plan P = kernel_plan(N);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int s = static_cast<int>(threadIdx.x) / P.t;
     const bool act = s < P.spb;  // threads past spb t (the last warp's tail) only join the barriers
@@ -534,7 +576,7 @@ namespace mixed_detail {
 template <int N>
 bool fill(int n, int dir, MixedLaunch *o) {
     if (n != N) return false;
-    constexpr Plan P = mixed_plan(N);
+    constexpr Plan P = kernel_plan(N);
     o->fn = dir < 0 ? reinterpret_cast<const void *>(&fft_mixed_kernel<N, -1>)
                     : reinterpret_cast<const void *>(&fft_mixed_kernel<N, 1>);
     o->threads = P.threads;

@@ -213,6 +213,22 @@ def test_fft_mixed_radix_vs_dft(bp, n):
         assert fft_rel_err(X, ref).max() <= tol(n), (n, direction)
 
 
+# radices 18, 20, 24 and 25 (each first and in the middle or last), several whole
+# blocks of signals and a ragged last one; the bound of every length
+@pytest.mark.parametrize("n", [324, 400, 432, 576, 600, 625, 2000, 3000, 6250, 12000])
+def test_fft_mixed_large_radices(bp, n):
+    batch = 19 if n < 1000 else 3
+    x = si.fft_c64(batch, n, stream=2500 + n)
+    for direction in (-1, 1):
+        # from 1000 points on the O(N^2) oracle takes too long
+        if n < 1000:
+            ref = oracle.dft(x, direction)
+        else:
+            z = x.astype(np.complex128)
+            ref = np.fft.fft(z, axis=1) if direction < 0 else np.fft.ifft(z, axis=1, norm="forward")
+        assert fft_rel_err(run_fft(bp, x, direction), ref).max() <= tol(n), (n, direction)
+
+
 def test_fft_mixed_radix_every_length(bp):
     """Every length with a compile-time kernel (all 2^a 3^b 5^c up to 12288
     that are not powers of two), both directions.  Below 1000 points: three
