@@ -1226,13 +1226,13 @@ def nonpow2_report(args):
         ms = timeit(lambda: bp.fft_batched(z, zo, n, batch, -1))
         tc = timeit(lambda: lib.extref_fft_c2c(ctypes.c_void_p(z.data_ptr()), ctypes.c_void_p(zo.data_ptr()), n, batch,
                                                -1, ctypes.c_void_p(st.cuda_stream)))
-        v = n
-        for f in (2, 3, 5):
+        v, prime = n, 1  # what is left of n, and its largest factor taken out
+        for f in (2, 3, 5, 7, 11, 13, 17, 19, 23, 29, 31):
             while v % f == 0:
-                v //= f
+                v, prime = v // f, f
         extra = {"cufft_ms": round(tc, 5), "ours_speedup_vs_cufft": round(tc / ms, 3)}
         if v == 1 and n <= 12288:
-            kind = "fft_mixed_radix"
+            kind = "fft_mixed_radix" if prime <= 5 else "fft_prime_radix"
         else:
             kind = "fft_bluestein"
             extra["inner_M"] = 1 << (2 * n - 2).bit_length()
