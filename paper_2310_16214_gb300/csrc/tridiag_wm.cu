@@ -188,9 +188,14 @@ __global__ void __launch_bounds__(MAXT, MINB)
             c[4 * q] = vc.x; c[4 * q + 1] = vc.y; c[4 * q + 2] = vc.z; c[4 * q + 3] = vc.w;
             d[4 * q] = vd.x; d[4 * q + 1] = vd.y; d[4 * q + 2] = vd.z; d[4 * q + 3] = vd.w;
         }
-        // the slot is read (and the exchange buffers of the last system too); on
-        // a timeout every thread leaves, the copy having been waited for
-        if (!__syncthreads_and(ok)) return;
+        // the slot is read (and the exchange buffers of the last system too)
+        if (!__syncthreads_and(ok)) {
+            // a wait ran out: the block leaves once its copies, one phase at most,
+            // have landed (or the second wait for them has run out too), because the
+            // slot may belong to another block afterwards
+            if (t == 0) mbar_wait_bounded(&full, parity);
+            return;
+        }
         if (t == 0 && sys + gridDim.x < batch) {
             fence_proxy_async();
             issue(sys + gridDim.x);
