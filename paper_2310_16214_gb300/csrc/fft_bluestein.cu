@@ -213,11 +213,13 @@ int tables_for(int64_t n, int dir, int logm, Tables *out) {
         cudaFree(t.h);
         return cuda_error(e, "Bluestein tables");
     }
-    if ((e = cudaMemcpy(t.h, h32.data(), n * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess ||
-        (e = cudaMemcpy(t.G, G32.data(), M * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess) {
+    int rc = upload(t.h, h32.data(), static_cast<size_t>(n) * sizeof(float2), "Bluestein tables upload");
+    if (rc == BPLG_OK)
+        rc = upload(t.G, G32.data(), static_cast<size_t>(M) * sizeof(float2), "Bluestein tables upload");
+    if (rc != BPLG_OK) {
         cudaFree(t.h);
         cudaFree(t.G);
-        return cuda_error(e, "Bluestein tables upload");
+        return rc;
     }
     g_tables[std::make_tuple(dev, n, dir)] = t;
     *out = t;

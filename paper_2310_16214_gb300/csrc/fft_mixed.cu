@@ -44,10 +44,10 @@ int table_for(int64_t n, const MixedLaunch &ml, const float2 **out) {
     float2 *d = nullptr;
     if ((e = cudaMalloc(&d, h.size() * sizeof(float2))) != cudaSuccess)
         return cuda_error(e, "mixed-radix twiddles");
-    if ((e = cudaMemcpy(d, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice)) !=
-        cudaSuccess) {
+    const int rc = upload(d, h.data(), h.size() * sizeof(float2), "mixed-radix twiddles upload");
+    if (rc != BPLG_OK) {
         cudaFree(d);
-        return cuda_error(e, "mixed-radix twiddles upload");
+        return rc;
     }
     g_tables[std::make_pair(dev, n)] = d;
     *out = d;

@@ -217,9 +217,10 @@ int entry_for(int64_t n, Entry *out) {
     if (h.empty()) h.push_back(make_float2(1.f, 0.f));  // one stage: no twiddles
     float2 *d = nullptr;
     if ((e = cudaMalloc(&d, h.size() * sizeof(float2))) != cudaSuccess) return cuda_error(e, "prime-radix twiddles");
-    if ((e = cudaMemcpy(d, h.data(), h.size() * sizeof(float2), cudaMemcpyHostToDevice)) != cudaSuccess) {
+    const int rc = upload(d, h.data(), h.size() * sizeof(float2), "prime-radix twiddles upload");
+    if (rc != BPLG_OK) {
         cudaFree(d);
-        return cuda_error(e, "prime-radix twiddles upload");
+        return rc;
     }
     *out = g_entries[std::make_pair(dev, n)] = Entry{p, d};
     return BPLG_OK;

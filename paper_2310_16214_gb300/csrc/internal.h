@@ -155,6 +155,9 @@ constexpr int kBluesteinMaxLog = 23;
 int fft_bluestein_launch(const bplg_plan *plan_m, const void *in, void *out, int64_t n, int64_t batch, int dir,
                          cudaStream_t s);
 
+// host memory to the device, on the device when it returns BPLG_OK (upload.cu)
+int upload(void *dst, const void *src, size_t bytes, const char *what);
+
 // twiddle table of the current device (layout: tw_root, tw_stage16 in fft_common.cuh; M = 2..2^14)
 int twiddles_for_current_device(const void **tw);
 

@@ -348,12 +348,10 @@ int uneven_create(const bplg_item *items, int64_t count, UnevenBatch **out) {
     if ((e = cudaMalloc(&ub->d_units, std::max<size_t>(1, h_units.size()) * sizeof(UnitDesc))) != cudaSuccess)
         return cuda_error(e, "uneven units");
     if ((e = cudaMalloc(&ub->d_counters, 4 * sizeof(int))) != cudaSuccess) return cuda_error(e, "uneven counters");
-    if ((e = cudaMemcpy(ub->d_items, h_items.data(), h_items.size() * sizeof(ItemDesc), cudaMemcpyHostToDevice)) !=
-        cudaSuccess)
-        return cuda_error(e, "uneven upload");
-    if (!h_units.empty() && (e = cudaMemcpy(ub->d_units, h_units.data(), h_units.size() * sizeof(UnitDesc),
-                                            cudaMemcpyHostToDevice)) != cudaSuccess)
-        return cuda_error(e, "uneven upload");
+    rc = upload(ub->d_items, h_items.data(), h_items.size() * sizeof(ItemDesc), "uneven upload");
+    if (rc == BPLG_OK && !h_units.empty())
+        rc = upload(ub->d_units, h_units.data(), h_units.size() * sizeof(UnitDesc), "uneven upload");
+    if (rc != BPLG_OK) return rc;
 
     const int fsm = fft_uneven_smem(), tsm = tri_uneven_smem();
     rc = ensure_smem_attr(reinterpret_cast<const void *>(&uneven_fft_kernel), fsm);
