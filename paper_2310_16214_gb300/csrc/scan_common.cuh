@@ -18,12 +18,16 @@
 
 namespace bplg {
 
-template <int P>
+// RUNS: P consecutive elements a thread all the same, one prefix for them.
+template <int P, bool RUNS = false>
 struct ScanRows {
-    static constexpr int V = P < 4 ? P : 4;
+    static constexpr int W = P < 4 ? P : 4;       // elements of one access
+    static constexpr int V = RUNS ? P : W;        // adjacent elements that share a prefix
     static constexpr int ROWS = P / V;
-    // first element of thread t's row q in its problem of tps threads
+    static constexpr int GROUPS = P / W;
+    // first element of thread t's access q in its problem of tps threads
     __device__ __forceinline__ static int pos(int t, int tps, int q) {
+        if (ROWS == 1) return t * P + q * W;
         return tps >= 32 ? (t >> 5) * (32 * P) + q * (32 * V) + (t & 31) * V : q * (tps * V) + t * V;
     }
 };
@@ -31,24 +35,25 @@ struct ScanRows {
 // The inclusive prefix of a problem whose elements its tps threads hold in v
 // as above: a power of two of threads up to 32, else whole warps (wl: this
 // thread's warp in the problem).  warp_tot: 32 elements of shared memory.
-template <typename E, int P, int PATTERN>
+template <typename E, int P, int PATTERN, bool RUNS = false>
 __device__ __forceinline__ void scan_problem(E (&v)[P], int tps, int wl, E *warp_tot) {
-    using S = ScanRows<P>;
+    using S = ScanRows<P, RUNS>;
     const int lane = threadIdx.x & 31;
     const int width = tps < 32 ? tps : 32;
     const int lane_in_seg = lane & (width - 1);
     E add[S::ROWS];  // what each row of the thread gets from the rows and lanes before it
-    E off = E(0);
+    E off = E(0);    // in the last lane of a segment finally the segment's total
 #pragma unroll
-    for (int q = 0; q < S::ROWS; ++q) {
+    for (int q = 0; q < S::ROWS; ++q)
 #pragma unroll
         for (int i = 1; i < S::V; ++i) v[S::V * q + i] += v[S::V * q + i - 1];
+#pragma unroll
+    for (int q = 0; q < S::ROWS; ++q) {
         const E incl = seg_scan<PATTERN>(v[S::V * q + S::V - 1], lane_in_seg, width);
         const E excl = __shfl_up_sync(kFullMask, incl, 1, width);
         add[q] = off + (lane_in_seg == 0 ? E(0) : excl);
-        off += __shfl_sync(kFullMask, incl, width - 1, width);
+        off += q + 1 < S::ROWS ? __shfl_sync(kFullMask, incl, width - 1, width) : incl;
     }
-    E before = E(0);
     if (tps > 32) {
         const int warp = threadIdx.x >> 5;
         if (lane == 31) warp_tot[warp] = off;
@@ -56,18 +61,18 @@ __device__ __forceinline__ void scan_problem(E (&v)[P], int tps, int wl, E *warp
         const int wps = tps >> 5;
         E w = (lane < wps) ? warp_tot[(warp - wl) + lane] : E(0);
         w = seg_scan<PATTERN>(w, lane, 32);
-        before = __shfl_sync(kFullMask, w, wl > 0 ? wl - 1 : 0);
+        E before = __shfl_sync(kFullMask, w, wl > 0 ? wl - 1 : 0);
         if (wl == 0) before = E(0);
+#pragma unroll
+        for (int q = 0; q < S::ROWS; ++q) add[q] += before;
     }
 #pragma unroll
-    for (int q = 0; q < S::ROWS; ++q) {
-        add[q] += before;
+    for (int q = 0; q < S::ROWS; ++q)
 #pragma unroll
         for (int i = 0; i < S::V; ++i) v[S::V * q + i] += add[q];
-    }
 }
 
-// One row of a thread: V elements at p, aligned to V elements.
+// One access of a thread: V elements at p, aligned to V elements.
 template <typename E, int V>
 __device__ __forceinline__ void load_row(const E *p, E *v) {
     E r[V];

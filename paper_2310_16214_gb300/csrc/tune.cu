@@ -329,11 +329,17 @@ ModelOp model_op(const bplg_plan &p, int64_t n) {
     switch (p.op) {
         case BPLG_OP_SCAN:
             m.bpe = 8;
-            m.instr = P * 2.0 + 16.0 * std::max(1, P / 4) + (tps > 32 ? 12 : 0);
             m.bars = tps > 32 ? 1 : 0;
             m.acc = 2.0 * std::max(1, P / 4);
-            m.lines = std::max<double>(std::min(P, 4), 0.75 * grouped_lines(tps, 4.0 * std::min(P, 4)));  // a problem's lanes adjacent
-            m.lsu = 7.0 * std::max(1, P / 4);                    // a shuffle prefix per row
+            if (scan_in_runs(p, n)) {
+                m.instr = P * 2.0 + 16.0 + (tps > 32 ? 12 : 0);
+                m.lines = warp_lines(P * 4.0, 16.0);
+                m.lsu = 7.0;
+            } else {
+                m.instr = P * 2.0 + 16.0 * std::max(1, P / 4) + (tps > 32 ? 12 : 0);
+                m.lines = std::max<double>(std::min(P, 4), 0.75 * grouped_lines(tps, 4.0 * std::min(P, 4)));  // a problem's lanes adjacent
+                m.lsu = 7.0 * std::max(1, P / 4);                    // a shuffle prefix per row
+            }
             break;
         case BPLG_OP_FFT:
         case BPLG_OP_FFT_TC: {

@@ -103,6 +103,45 @@ def test_tridiag_cr_plan_needs_power_of_two(bp):
         run_tri(bp, sysm, bp.make_plan(bp.OP_TRIDIAG, 128, 2, 1, cr_switch=32, shuffle=1))
 
 
+# Both forms of the kernel for rows (on the threads the row needs, and padded)
+# under every plan, at lengths on both sides of the lines between them.
+@pytest.mark.parametrize("n", [6, 12, 15, 20, 28, 60, 63, 65, 96, 127, 130, 255, 260, 448, 500, 511, 640, 700, 1020, 2000])
+def test_scan_row_forms_every_plan(bp, n):
+    batch = 67
+    x = si.scan_i32(batch, n, stream=1500 + n)
+    ref = oracle.scan_i32(x)
+    f = si.scan_f32(batch, n, stream=1600 + n, integer_valued=True)  # sums exact in float32
+    for p in bp.enumerate_plans(bp.OP_SCAN, bp.I32, next_pow2(n)) + [None]:
+        assert np.array_equal(run_scan(bp, x, p), ref), p
+    for p in bp.enumerate_plans(bp.OP_SCAN, bp.F32, next_pow2(n))[::7] + [None]:
+        assert np.array_equal(run_scan(bp, f, p), np.cumsum(f.astype(np.float64), axis=1).astype(np.float32)), p
+
+
+# A row a little longer than a power of two costs about what that one costs per
+# element (0.98 of it; 1.24 to 1.36 when every four elements had a prefix of their own).
+@pytest.mark.parametrize("n", [260, 300])
+def test_scan_short_rows_keep_the_rate(bp, n):
+    total = 1 << 26
+    x = torch.zeros(total, dtype=torch.int32, device="cuda")
+    y = torch.empty_like(x)
+
+    def per_element(m, plan):
+        ts = []
+        for _ in range(6):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(10):
+                bp.scan_batched(x, y, m, total // m, plan=plan)
+            e1.record()
+            e1.synchronize()
+            ts.append(e0.elapsed_time(e1) / (total // m * m))
+        return min(ts)
+
+    whole = per_element(256, None)
+    for plan in (None, bp.make_plan(bp.OP_SCAN, 512, P=16, spb=2)):
+        assert per_element(n, plan) <= 1.15 * whole, plan
+
+
 # Rows that start 1, 2 and 3 elements past a 16-byte boundary, at lengths
 # whose last thread, warp or block is nearly empty or exactly full, and at the
 # longest odd lengths (no room for the shift at n = 32767); in place too.
