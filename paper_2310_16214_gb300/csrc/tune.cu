@@ -280,6 +280,8 @@ int analytic_plan(int op, int dtype, int64_t n, bplg_plan *out) {
 //   issue            4        warp instructions per clock per SM
 //   line             1        clock per 128-byte line of a warp-wide access
 //   FP64             2        fused multiply-adds per clock per SM
+//   flight           4 %      of bandwidth per 64 KB that an SM's threads request beyond the first 64 KB (scan; at
+//                             2^26 elements, n = 1024: P = 8 64 KB 78.0 us, 16 80 KB 79.4, 32 128 KB 80.0)
 //   clock, bandwidth 0.92 x the peak SM clock, 0.83 x the nominal HBM rate
 //                    (what sustained streaming reaches)
 // A pipelined plan (bulk-copy ring) hides half the latency.
@@ -292,6 +294,7 @@ constexpr double kModelBlockLaunch = 80e-9;
 constexpr double kModelIpc = 4.0;
 constexpr double kModelLine = 1.0;
 constexpr double kModelFp64PerClk = 2.0;
+constexpr double kModelFlight = 0.04;
 constexpr double kModelNorm = 4.0;
 
 struct ModelOp {
@@ -303,6 +306,7 @@ struct ModelOp {
     double lsu = 0;     // further 128-byte wavefronts of a warp in the load/store unit (exchanges, twiddles)
     bool piped = false; // bulk-copy ring in front of the loads
     bool persistent = false;  // one block per SM looping over tiles, the next tile's loads in flight
+    double flight = 0;  // bytes a thread has requested at once
     double fp64 = 0;    // FP64 pipe operations per element
 };
 
@@ -331,6 +335,7 @@ ModelOp model_op(const bplg_plan &p, int64_t n) {
             m.bpe = 8;
             m.bars = tps > 32 ? 1 : 0;
             m.acc = 2.0 * std::max(1, P / 4);
+            m.flight = 4.0 * P;
             if (scan_in_runs(p, n)) {
                 m.instr = P * 2.0 + 16.0 + (tps > 32 ? 12 : 0);
                 m.lines = warp_lines(P * 4.0, 16.0);
@@ -473,7 +478,8 @@ double model_kernel(const ModelOp &m, const DevModel &dm, int64_t elems, int64_t
                                       : per_sm_blocks * res / b_a;
     const double terms[6] = {
         t_lat,                                                            // latency, b_a blocks (tiles) in flight
-        static_cast<double>(elems) * m.bpe / dm.bw,                       // HBM bandwidth
+        static_cast<double>(elems) * m.bpe / dm.bw *                      // HBM bandwidth
+            (1.0 + kModelFlight * std::max(0.0, b_a * threads * m.flight / 65536.0 - 1.0)),
         per_sm_blocks * wpb * m.instr / (kModelIpc * dm.clk),             // issue
         per_sm_blocks * wpb * (m.acc * m.lines + m.lsu) * kModelLine / dm.clk,  // load/store unit
         (m.persistent ? 1.0 : per_sm_blocks) * kModelBlockLaunch,         // block launches
