@@ -125,7 +125,7 @@ int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64
     if (np == n || plan)
         rc = resolve_plan(BPLG_OP_SCAN, dtype, np, batch, plan, &p, np == n ? &tk : nullptr);
     else if (!cache_lookup(BPLG_OP_SCAN, dtype, np, batch, &p))  // a tuned plan of n', else the ragged rule's
-        p = scan_ragged_plan(n);
+        p = scan_ragged_plan(n, batch);
     if (rc != BPLG_OK) return rc;
     p.n = static_cast<int32_t>(np);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);

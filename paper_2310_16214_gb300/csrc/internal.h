@@ -55,7 +55,7 @@ int check_grid(int64_t blocks, const char *what);
 
 // ---- per-op kernel tables (each returns false if the plan has no kernel)
 bool scan_launch_info(const bplg_plan &p, int dtype, int64_t n, int64_t batch, Launch *out);
-bplg_plan scan_ragged_plan(int64_t n);
+bplg_plan scan_ragged_plan(int64_t n, int64_t batch);
 bool scan_in_runs(const bplg_plan &p, int64_t n);  // P consecutive elements a thread
 int scan_launch(const bplg_plan &p, int dtype, const void *in, void *out, int64_t n, int64_t batch,
                 cudaStream_t s);

@@ -235,39 +235,58 @@ static RaggedForm ragged_form(int64_t n, int P) {
 }
 
 // The plan of a length n that is not a power of two when the caller gives none.
-// Multiples of 4 from 16 to 512: P = 16 above 128 where n is less than three quarters
-// of n', else 8 (padded form; 2^26 int32 elements, P = 16 / P = 8 / rows at P = 32: n
-// = 28 84 / 79 / 82 us, 100 80 / 78 / 79, 260 78 / 95 / 102, 320 78 / 86 / 88, 500 84 /
-// 78 / 80).  Others: the P whose threads are idle least (a row of 1100 elements fills
-// 86 % of the warps it takes at P = 8, 54 % at P = 32: 0.0480 against 0.0585 ms, 2^25
-// elements), the larger one of equals, but 16 for rows off boundaries below 128 (65:
-// 0.0580 against 0.0607) or without the elements before them (255: 0.0476 against
-// 0.0620).  Below 16 the accesses are element-wise: P = 4 where that leaves few elements
-// over (7: 0.092 against 0.121 at 2^26), else 8 (6: 0.085 against 0.101).  Blocks of
-// about 64 threads, so that a barrier holds up few (128 below 16 elements and with the
-// padded P = 8).
-bplg_plan scan_ragged_plan(int64_t n) {
+//   - Below 16 elements the accesses are element-wise: P = 4 where that leaves few
+//     elements over (7: 0.092 against 0.121 ms at 2^26), else 8 (6: 0.085 against 0.101).
+//   - Up to 2^20 elements in all the call is as long as one block: P = 8, the least
+//     serial work that 1024 threads allow (16 from n = 8190 on, where the elements before
+//     a row would not fit), in blocks of 128 threads or more.  Microseconds on the
+//     device at 2^16 elements, P = 8 / 32: n = 800 1.5 / 3.0, 2000 1.9 / 3.3, 5000 2.4 / 3.4.
+//   - Multiples of 4 up to 1020: P = 16 from 132 to 380 where n is less than three
+//     quarters of n', 32 from 384 to 444 in large batches, else 8 (2^26 int32 elements, P =
+//     16 / P = 8 / rows at P = 32: n = 28 84 / 79 / 82 us, 100 80 / 78 / 79, 260 78 / 95 /
+//     102, 320 78 / 86 / 88, 400 82 / 83 / 80, 500 84 / 78 / 80, 800 82 / 82 / 80), blocks
+//     of 128 threads with P = 8.
+//   - Others: the P whose threads are idle least (a row of 1100 elements fills 86 % of
+//     the warps it takes at P = 8, 54 % at P = 32: 0.0480 against 0.0585 ms, 2^25
+//     elements), the larger one of equals; 32 only from 2^24 elements in all (n = 2000 at
+//     2^22 6.0 us, with 16 5.6; 3000 at 2^25 44 us, 46) and where it has the elements before
+//     the row (255: 62 us at 2^25, with 16 48), 128 or more off boundaries (65: 0.0607
+//     against 0.0580).
+// Blocks of about 64 threads otherwise, so that a barrier holds up few.
+bplg_plan scan_ragged_plan(int64_t n, int64_t batch) {
     const int64_t np = next_pow2(n);
-    int best = n < 16 && (np == 4 || 5 * n > 4 * np) ? 4 : 8;
-    double best_use = 0.0;
-    for (int P = 32; P >= 8 && n >= 16; P /= 2) {
-        const RaggedForm f = ragged_form(n, P);
-        if (np / P > 1024 || (P == 32 && n % 4 != 0 && (n < 128 || f.max_shift == 0))) continue;
-        const double use = static_cast<double>(n) / (static_cast<double>(P) * f.tps);
-        if (use > best_use * 1.05) {
-            best = P;
-            best_use = use;
+    const bool small = batch <= (int64_t(1) << 20) / n, large = batch >= (int64_t(1) << 24) / n;
+    int best = 8, threads = 64;
+    if (n < 16) {
+        best = np == 4 || 5 * n > 4 * np ? 4 : 8;
+        threads = 128;
+    } else if (small) {
+        while (best < 32 && (np / best > 1024 || ragged_form(n, best).tps > 1024)) best *= 2;
+        threads = 128;
+    } else if (n % 4 == 0 && n < 1024) {
+        const bool wide = np == 256 || np == 512, full = 4 * n >= 3 * np;
+        best = wide && !full ? 16 : (np == 512 && n < 448 && large ? 32 : 8);
+        if (best == 8) threads = 128;
+    } else {
+        double best_use = 0.0;
+        for (int P = 32; P >= 8; P /= 2) {
+            const RaggedForm f = ragged_form(n, P);
+            if (np / P > 1024) continue;
+            if (P == 32 && np <= 16384 && (!large || (n % 4 != 0 && (n < 128 || f.max_shift == 0)))) continue;
+            const double use = static_cast<double>(n) / (static_cast<double>(P) * f.tps);
+            if (use > best_use * 1.05) {
+                best = P;
+                best_use = use;
+            }
         }
     }
-    const bool narrow = n % 4 == 0 && n >= 16 && n <= 512;
-    if (narrow) best = n > 128 && 4 * n < 3 * np ? 16 : 8;
     bplg_plan p = {};
     p.op = BPLG_OP_SCAN;
     p.n = static_cast<int32_t>(np);
     p.P = best;
     p.radix = 2;
     p.shuffle = 1;
-    p.spb = std::max(1, (n < 16 || (narrow && best == 8) ? 128 : 64) / ragged_form(n, p.P).tps);
+    p.spb = std::max(1, threads / ragged_form(n, p.P).tps);
     p.L = static_cast<int32_t>(p.spb * (np / p.P));
     plan_finalize(&p, BPLG_I32, np);
     return p;

@@ -142,6 +142,44 @@ def test_scan_short_rows_keep_the_rate(bp, n):
         assert per_element(n, plan) <= 1.15 * whole, plan
 
 
+# The plan of a call without one depends on the batch: a small, a middle and a large
+# one of each kind of length.
+@pytest.mark.parametrize("n", [20, 33, 130, 260, 400, 500, 800, 1000, 1100, 2000, 5000, 5001, 8191, 9000, 20000, 32767])
+def test_scan_default_plan_by_batch(bp, n):
+    for total in (1 << 19, 3 << 20, (1 << 24) + n):
+        batch = total // n
+        x = torch.randint(-1000, 1001, (batch, n), dtype=torch.int32, device="cuda")
+        y = torch.empty_like(x)
+        bp.scan_batched(x, y, n, batch)
+        assert torch.equal(y, torch.cumsum(x, dim=1, dtype=torch.int32)), total
+
+
+# A few rows take about as long as a few of the next power of two (1.0 to 1.1 of it on
+# the device; 1.6 to 1.7 when 32 elements a thread were taken there too).
+@pytest.mark.parametrize("n", [1000, 2000])
+def test_scan_few_rows(bp, n):
+    x = torch.zeros(1 << 16, dtype=torch.int32, device="cuda")
+    y = torch.empty_like(x)
+
+    def per_call(m):
+        bp.scan_batched(x, y, m, 16)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            for _ in range(50):
+                bp.scan_batched(x, y, m, 16)
+        ts = []
+        for _ in range(6):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            g.replay()
+            e1.record()
+            e1.synchronize()
+            ts.append(e0.elapsed_time(e1))
+        return min(ts)
+
+    assert per_call(n) <= 1.3 * per_call(next_pow2(n))
+
+
 # Rows that start 1, 2 and 3 elements past a 16-byte boundary, at lengths
 # whose last thread, warp or block is nearly empty or exactly full, and at the
 # longest odd lengths (no room for the shift at n = 32767); in place too.
