@@ -204,7 +204,7 @@ int bplg_tridiag_batched(const float *a, const float *b, const float *c, const f
     // without a plan (given or tuned for n') the longer ones take the persistent
     // bulk-copy form of it
     bplg_plan p;
-    if (!plan && tridiag_wm_tma_applies(n) && !cache_lookup(BPLG_OP_TRIDIAG_WM, BPLG_F32, np, batch, &p))
+    if (!plan && tridiag_wm_tma_applies(n, batch) && !cache_lookup(BPLG_OP_TRIDIAG_WM, BPLG_F32, np, batch, &p))
         return tridiag_wm_tma_launch(a, b, c, d, x, n, batch, static_cast<cudaStream_t>(stream));
     const int op = np != n || (plan && plan->op == BPLG_OP_TRIDIAG_WM) ? BPLG_OP_TRIDIAG_WM : BPLG_OP_TRIDIAG;
     OnlineTicket tk;

@@ -86,7 +86,7 @@ bool tridiag_wm_launch_info(const bplg_plan &p, int64_t n, int64_t batch, Launch
 int tridiag_wm_launch(const bplg_plan &p, const float *a, const float *b, const float *c, const float *d, float *x,
                       int64_t n, int64_t batch, cudaStream_t s);
 // its persistent bulk-copy form for lengths that are not powers of two
-bool tridiag_wm_tma_applies(int64_t n);
+bool tridiag_wm_tma_applies(int64_t n, int64_t batch);
 int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const float *d, float *x, int64_t n,
                           int64_t batch, cudaStream_t s);
 int tridiag_refined_launch(const bplg_plan &p, const float *a, const float *b, const float *c,

@@ -299,15 +299,23 @@ int tridiag_wm_device_status(int *flag, bool reset) {
     return BPLG_OK;
 }
 
-// Which lengths take it: those above 256 whose padded form wastes threads or has
-// rows off 16-byte boundaries.  Up to 1024 a multiple of 4 within 1/16 of the
-// power of two is as fast padded (P = 8, whose lanes lie closer): n = 500 0.0556
-// ms against 0.0566, 1000 0.0580 against 0.0600; up to 256 a block here is one
-// warp with half of its lanes idle.
-bool tridiag_wm_tma_applies(int64_t n) {
+// Which calls take it: lengths above 256 whose padded form wastes threads or has
+// rows off 16-byte boundaries, unless
+//   - a multiple of 4 above three quarters of the power of two, up to 2048: of the
+//     padded form's threads (P = 8) nearly all are busy, and without a slot in shared
+//     memory more of its blocks fit an SM (2^24 unknowns, padded / bulk copies: n = 400
+//     60 / 66 us, 800 64 / 76, 1600 62 / 72, 2000 58 / 67, but 768 66 / 61, 1500 66 / 59,
+//     4000 74 / 74); up to 256 a block here is one warp with half of its lanes idle;
+//   - few systems, which take as long as one, the longer the more equations a thread
+//     has (device time, padded / bulk copies: 76 systems of n = 300 2.5 / 3.2 us, 491 2.6
+//     / 3.7, 1100 3.2 / 3.7, 3600 4.6 / 5.4, but 1025 4.4 / 3.7, 6500 6.8 / 6.5; the two
+//     meet at 2400 systems of 300, 900 of 600, 600 of 1500, 300 of 2200, 300 of 641, 150
+//     of 901).
+bool tridiag_wm_tma_applies(int64_t n, int64_t batch) {
     if (is_pow2(n) || n <= 256 || n > (int64_t(1) << kTridiagMaxLog)) return false;
-    const int64_t np = next_pow2(n);
-    return n % 4 != 0 || n > 1024 || (np - n) * 16 > np;
+    const int64_t few = n % 4 == 0 ? (n <= 384 ? 2432 : (n <= 2048 ? 608 : (n <= 4096 ? 152 : 0)))
+                                   : (n <= 640 ? 304 : (n <= 900 ? 152 : 0));
+    return batch > few && (n % 4 != 0 || n > 2048 || 4 * n <= 3 * next_pow2(n));
 }
 
 int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const float *d, float *x, int64_t n,

@@ -215,6 +215,48 @@ def test_tridiag_rows_off_alignment(bp, n, batch):
     assert bp.device_status() == 0
 
 
+# The bulk-copy solver and the padded one take turns over length and batch: both
+# sides of each line, every shape of the bulk-copy solver in batches large enough for it.
+@pytest.mark.parametrize("n,batch", [(380, 2433), (384, 2432), (384, 2433), (388, 700), (385, 304), (385, 305), (637, 310),
+                                     (640, 609), (641, 152), (641, 153), (768, 608), (768, 609), (772, 700), (900, 160),
+                                     (901, 2), (1500, 609), (1536, 609), (1540, 620), (2044, 609), (2052, 152), (2052, 153),
+                                     (4092, 153), (4100, 1)])
+def test_tridiag_ragged_lines(bp, n, batch):
+    a, b, c, d, _ = si.tridiag_f32(batch, n, stream=1900 + n)
+    a[:, 0] = np.nan  # never read
+    c[:, -1] = np.nan
+    rows = np.unique(np.r_[:3, batch // 2, max(0, batch - 3):batch])
+    rows = rows[rows < batch]
+    x = run_tri(bp, (a, b, c, d))
+    assert np.all(np.isfinite(x))
+    assert tri_rel_err(x[rows], oracle.thomas(a[rows], b[rows], c[rows], d[rows])).max() <= 1e-4
+    assert bp.device_status() == 0
+
+
+# Lengths whose padded form is the faster one take it without a plan (the bulk copies
+# took 1.16 to 1.19 of its time).
+@pytest.mark.parametrize("n", [800, 2000])
+def test_tridiag_ragged_as_fast_as_padded(bp, n):
+    total = 1 << 24
+    ts = [torch.zeros(total, device="cuda") for _ in range(5)]
+    ts[1].fill_(1.0)
+
+    def per_unknown(m, plan):
+        best = []
+        for _ in range(6):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(10):
+                bp.tridiag_batched(*ts, m, total // m, plan=plan)
+            e1.record()
+            e1.synchronize()
+            best.append(e0.elapsed_time(e1))
+        return min(best) / (total // m * m)
+
+    padded = bp.query_plan(bp.OP_TRIDIAG_WM, bp.F32, next_pow2(n), total // n)
+    assert per_unknown(n, None) <= 1.08 * per_unknown(n, padded)
+
+
 # ------------------------------------------------------------------- FFT ----
 
 def tol(n):
