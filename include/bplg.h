@@ -37,8 +37,11 @@
  *     errors are reported before anything is enqueued.
  *   - Plans: a NULL plan means "the plan bplg_query_plan returns" (with
  *     online tuning on, a candidate of the online search instead; see
- *     bplg_set_online_tuning).  A non-NULL plan is validated against the size
- *     and the device; an unusable plan returns BPLG_ERR_INVALID_PLAN without
+ *     bplg_set_online_tuning).  bplg_query_plan and the tuner know powers of
+ *     two; what a NULL plan means at other lengths is said at each entry
+ *     point, and a plan tuned for the next power of two is used there when
+ *     the caller passes it, or by a solve that runs that length's kernel
+ *     padded.  A non-NULL plan is validated against the size and the device; an unusable plan returns BPLG_ERR_INVALID_PLAN without
  *     launching.
  */
 #ifndef BPLG_H
@@ -161,9 +164,9 @@ typedef struct {
  *   in,out device, [batch][n] of dtype; in == out (in place) is allowed.
  *   n      1 <= n <= 32768; batch >= 1.  A power of two runs its own plan;
  *          any other n runs a plan of the next power of two n' (plan->n ==
- *          n'; plan NULL: the tuned plan of n' if there is one, else one
- *          chosen for n itself), the rows read as if padded with zeros to n'
- *          (rows stay n apart, nothing outside a row is read or written).
+ *          n'; plan NULL: one chosen for n and batch), the rows read as if
+ *          padded with zeros to n' (rows stay n apart, nothing outside a row
+ *          is read or written).
  * Errors: INVALID_ARG, UNSUPPORTED_SIZE, INVALID_PLAN, CUDA. */
 int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64_t batch,
                       const bplg_plan *plan, void *stream);
@@ -279,8 +282,8 @@ int bplg_fft_batched_noalloc(const void *in, void *out, int64_t n, int64_t batch
  *           n' (a BPLG_OP_TRIDIAG_WM plan with plan->n == n', or NULL): the
  *           system is padded with identity rows (a = c = 0, b = 1, d = 0),
  *           c[s][n-1] is taken as 0, rows stay n apart and nothing past n is
- *           written.  With plan NULL and no tuned plan of n' most such n
- *           above 256 run a persistent form of the solver with its own tiling,
+ *           written.  With plan NULL most such n above 256, in all but small
+ *           batches, run a persistent form of the solver with its own tiling,
  *           fed by bulk copies in whole 16-byte units: up to three elements on
  *           either side of a row may be read, none outside the arrays.
  * No pivoting: the systems must be safe for elimination without pivoting

@@ -257,6 +257,23 @@ def test_tridiag_ragged_as_fast_as_padded(bp, n):
     assert per_unknown(n, None) <= 1.08 * per_unknown(n, padded)
 
 
+# Tuning the next power of two does not change what a call of another length runs: the
+# same bits before and after.
+def test_ragged_calls_do_not_follow_the_tuned_power_of_two(bp):
+    n, batch = 3001, 700
+    a, b, c, d, _ = si.tridiag_f32(batch, n, stream=77)
+    before = run_tri(bp, (a, b, c, d))
+    bp.tune_plan(bp.OP_TRIDIAG_WM, bp.F32, next_pow2(n), batch, bp.TUNE_MODEL)
+    assert np.array_equal(run_tri(bp, (a, b, c, d)), before)
+    for n, batch in [(1000, 40), (1003, 20000), (5000, 3400)]:
+        x = torch.rand(batch, n, device="cuda") - 0.5
+        y0, y1 = torch.empty_like(x), torch.empty_like(x)
+        bp.scan_batched(x, y0, n, batch)
+        bp.tune_plan(bp.OP_SCAN, bp.F32, next_pow2(n), batch, bp.TUNE_EXHAUSTIVE)
+        bp.scan_batched(x, y1, n, batch)
+        assert torch.equal(y0, y1), n
+
+
 # ------------------------------------------------------------------- FFT ----
 
 def tol(n):
