@@ -41,8 +41,8 @@
  *     two; what a NULL plan means at other lengths is said at each entry
  *     point, and a plan tuned for the next power of two is used there when
  *     the caller passes it, or by a solve that runs that length's kernel
- *     padded.  A non-NULL plan is validated against the size and the device; an unusable plan returns BPLG_ERR_INVALID_PLAN without
- *     launching.
+ *     padded.  A non-NULL plan is validated against the size and the device;
+ *     an unusable plan returns BPLG_ERR_INVALID_PLAN without launching.
  */
 #ifndef BPLG_H
 #define BPLG_H
@@ -209,8 +209,8 @@ int bplg_fft_batched(const void *in, void *out, int64_t n, int64_t batch, int32_
 /* The same FFT with its DFT stages run on tensor cores as real contractions
  * on 16-bit operands split into hi and lo parts, x = xh + xl and
  * F = Fh + Fl, summing xh Fh + xh Fl + xl Fh in float32.
- *   io 0 (n >= 1024): every radix-16 stage; each 16-point DFT is a 32 x 32
- *        contraction issued as tcgen05.mma with the accumulator in tensor
+ *   io 0 (spb 4 at n = 512): every radix-16 stage; each 16-point DFT is a 32
+ *        x 32 contraction issued as tcgen05.mma with the accumulator in tensor
  *        memory; a mixed-radix first stage (log2 n not a multiple of 4)
  *        runs on the CUDA cores.
  *   io 1: the same stages in the legacy mma.sync m16n8k16 form.
@@ -227,8 +227,7 @@ int bplg_fft_batched(const void *in, void *out, int64_t n, int64_t batch, int32_
  *             exactly, and undoes it at the end).
  *   n        power of two, 512 <= n <= 16384; in, out as bplg_fft_batched.
  *   plan     op BPLG_OP_FFT_TC (radix 16; P, spb, io as above), or NULL
- *            (the GB300 cost model's choice; at n = 512, untuned, the io 0
- *            kernel, which the plan space offers from 1024 points on).
+ *            (the GB300 cost model's choice).
  * Errors: INVALID_ARG, UNSUPPORTED_SIZE, INVALID_PLAN, CUDA. */
 int bplg_fft_tc_batched(const void *in, void *out, int64_t n, int64_t batch, int32_t dir,
                         int32_t precision, const bplg_plan *plan, void *stream);
@@ -403,7 +402,9 @@ double bplg_phi(const double *efficiencies, int32_t count);
 /* All valid plans for (op, dtype, n) on the current device, in the library's
  * canonical order (written up to `capacity`; *count gets the total).
  * Validity uses the device limits and each kernel's register count from
- * cudaFuncGetAttributes.  Errors: INVALID_ARG, UNSUPPORTED_SIZE, CUDA. */
+ * cudaFuncGetAttributes.  One is not listed, though the tuners time it and
+ * bplg_query_plan returns it: the io 0 plan of the 512-point tensor-core FFT.
+ * Errors: INVALID_ARG, UNSUPPORTED_SIZE, CUDA. */
 int bplg_enumerate_plans(int32_t op, int32_t dtype, int64_t n, bplg_plan *out, int32_t capacity,
                          int32_t *count);
 

@@ -176,11 +176,8 @@ int bplg_fft_tc_batched(const void *in, void *out, int64_t n, int64_t batch, int
     if (!aligned16(in) || !aligned16(out)) return set_error(BPLG_ERR_INVALID_ARG, "fft tc: buffers must be 16-byte aligned");
     bplg_plan p;
     OnlineTicket tk;
-    const bool untuned512 = !plan && n == 512 && !cache_lookup(BPLG_OP_FFT_TC, BPLG_F32, n, batch, &p);
     int rc = resolve_plan(BPLG_OP_FFT_TC, BPLG_F32, n, batch, plan, &p, &tk);
     if (rc != BPLG_OK) return rc;
-    if (untuned512 && !tk.applies)
-        return fft_tc512_launch(in, out, batch, dir, precision, static_cast<cudaStream_t>(stream));
     const cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (tk.e0) cudaEventRecord(tk.e0, s);
     rc = fft_tc_launch(p, in, out, n, batch, dir, precision, s);
@@ -299,6 +296,9 @@ int bplg_enumerate_plans(int32_t op, int32_t dtype, int64_t n, bplg_plan *out, i
     std::vector<bplg_plan> plans;
     int rc = device_space(op, dtype, n, &plans, nullptr, nullptr);
     if (rc != BPLG_OK) return rc;
+    // the tcgen05 plan of 512 points is the tuners' (and the default) but not listed here
+    if (op == BPLG_OP_FFT_TC && n == 512)
+        plans.erase(std::remove_if(plans.begin(), plans.end(), [](const bplg_plan &p) { return p.io == 0; }), plans.end());
     *count = static_cast<int32_t>(plans.size());
     for (int i = 0; i < capacity && i < static_cast<int>(plans.size()); ++i) out[i] = plans[i];
     return BPLG_OK;

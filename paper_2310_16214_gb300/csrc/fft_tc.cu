@@ -485,8 +485,12 @@ __global__ void __launch_bounds__(MAXT)
 
 namespace {
 
+// 512 points: blocks of one tile of 128 butterflies a stage, four signals.  Measured at
+// 2^25 points against the mma.sync kernel's fastest plan: 0.500 -> 0.134 ms.
 template <int PREC, int DIR, int MAXT>
 const void *tc5_func_t(int logn) {
+    if constexpr (MAXT == 512)
+        if (logn == 9) return reinterpret_cast<const void *>(&fft_tc5_kernel<PREC, 9, DIR, MAXT>);
     switch (logn) {
         case 10: return reinterpret_cast<const void *>(&fft_tc5_kernel<PREC, 10, DIR, MAXT>);
         case 11: return reinterpret_cast<const void *>(&fft_tc5_kernel<PREC, 11, DIR, MAXT>);
@@ -561,30 +565,6 @@ int fft_tc_launch(const bplg_plan &p, const void *in, void *out, int64_t n, int6
     cudaError_t e = cudaLaunchKernel(li.func, dim3(static_cast<unsigned>(li.blocks)), dim3(li.threads), args,
                                      static_cast<size_t>(li.smem), s);
     return e == cudaSuccess ? BPLG_OK : launch_error(e, "fft tc launch", li.func, li.blocks, li.threads, li.smem);
-}
-
-// 512 points without a plan: the tcgen05 kernel with four signals in a block, one
-// tile of 128 butterflies a stage.  (The plan space offers that kernel from 1024
-// points on; at 512 its only plans run the mma.sync form.)  Measured at 2^25
-// points: 0.500 -> 0.134 ms.
-int fft_tc512_launch(const void *in, void *out, int64_t batch, int dir, int prec, cudaStream_t s) {
-    const void *f = prec == BPLG_TC_BF16 ? (dir < 0 ? reinterpret_cast<const void *>(&fft_tc5_kernel<BPLG_TC_BF16, 9, -1, 512>)
-                                                    : reinterpret_cast<const void *>(&fft_tc5_kernel<BPLG_TC_BF16, 9, 1, 512>))
-                                         : (dir < 0 ? reinterpret_cast<const void *>(&fft_tc5_kernel<BPLG_TC_F16, 9, -1, 512>)
-                                                    : reinterpret_cast<const void *>(&fft_tc5_kernel<BPLG_TC_F16, 9, 1, 512>));
-    int spb = 4, logn = 9;
-    const int threads = 128, smem = fft_tc_smem_bytes(512, spb, 0);
-    const int64_t blocks = (batch + spb - 1) / spb;
-    int rc = check_grid(blocks, "fft tc");
-    if (rc != BPLG_OK) return rc;
-    const void *tw = nullptr;
-    rc = twiddles_for_current_device(&tw);
-    if (rc == BPLG_OK) rc = ensure_smem_attr(f, smem);
-    if (rc != BPLG_OK) return rc;
-    void *args[] = {(void *)&in, (void *)&out, (void *)&tw, &logn, &spb, &batch};
-    cudaError_t e = cudaLaunchKernel(f, dim3(static_cast<unsigned>(blocks)), dim3(threads), args,
-                                     static_cast<size_t>(smem), s);
-    return e == cudaSuccess ? BPLG_OK : launch_error(e, "fft tc launch", f, blocks, threads, smem);
 }
 
 // Read (and optionally clear) the device error word of this file's kernels

@@ -64,7 +64,6 @@ bool fft_launch_info(const bplg_plan &p, int64_t n, int64_t batch, int dir, Laun
 int fft_launch(const bplg_plan &p, const void *in, void *out, int64_t n, int64_t batch, int dir,
                cudaStream_t s);
 
-int fft_tc512_launch(const void *in, void *out, int64_t batch, int dir, int prec, cudaStream_t s);
 int fft_tc_launch(const bplg_plan &p, const void *in, void *out, int64_t n, int64_t batch, int dir, int prec,
                   cudaStream_t s);
 

@@ -126,8 +126,8 @@ bool plan_structurally_valid(const bplg_plan &p, int dtype, int64_t n, std::stri
             if (p.smem_pad != 1 || p.smem_layout != 0 || p.io < 0 || p.io > 2)
                 return fail(why, "tensor-core FFT: padded interleaved layout; io 0 (tcgen05), 1 (mma.sync) or 2 "
                                  "(two GEMM passes)");
-            if (p.io == 0 && (n < 1024 || n > 16384 || p.L % 128 != 0))
-                return fail(why, "tensor-core FFT with tcgen05: 1024 <= n <= 16384 and blocks of 128-thread tiles");
+            if (p.io == 0 && (p.L % 128 != 0 || (n == 512 && p.L != 128)))
+                return fail(why, "tensor-core FFT with tcgen05: blocks of 128-thread tiles, one tile (spb 4) at n = 512");
             return true;
         case BPLG_OP_TRIDIAG_WM:
             if (n < 2) return fail(why, "Wang-Mou: n >= 2");

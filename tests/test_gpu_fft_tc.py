@@ -63,6 +63,27 @@ def test_default_512_runs_tcgen05(bp, batch):
     assert bp.device_status() == 0
 
 
+def test_512_tunes_to_tcgen05(bp):
+    """The tuners time the tcgen05 kernel at 512 points too: what they leave in
+    the cache is what a call without a plan ran before, and the plan that
+    query_plan names can be passed."""
+    batch = 1 << 14
+    z = si.fft_c64(batch, 512, stream=690)
+    plan = bp.query_plan(bp.OP_FFT_TC, bp.F32, 512, batch)
+    assert (plan.io, plan.spb, plan.L) == (0, 4, 128)
+    before = run(bp, z, -1, 1)
+    assert np.array_equal(run(bp, z, -1, 1, plan).view(np.uint32), before.view(np.uint32))
+    tuned, _ = bp.tune_plan(bp.OP_FFT_TC, bp.F32, 512, batch, bp.TUNE_EXHAUSTIVE)
+    assert tuned.key() == plan.key()
+    assert np.array_equal(run(bp, z, -1, 1).view(np.uint32), before.view(np.uint32))
+    rows = sample_rows(batch, k=24)
+    assert fft_rel_err(before[rows], oracle.fft(z[rows], -1)).max() <= 1e-5 * 9
+    with pytest.raises(bp.BplgError) as e:  # two tiles a block: no such plan at 512
+        bp.fft_tc_batched(c64_to_dev(z), c64_to_dev(z), 512, batch, -1, precision=1,
+                          plan=bp.make_plan(bp.OP_FFT_TC, 512, P=16, spb=8, io=0, radix=16, smem_pad=1))
+    assert e.value.code == bp.ERR_INVALID_PLAN
+
+
 @pytest.mark.parametrize("n", [1024, 4096, 16384])
 def test_precision_configuration_sampled(bp, n):
     # batch = 2^26 / N signals, default plan, both precisions
