@@ -365,6 +365,30 @@ def test_fft_mixed_large_radices(bp, n):
         assert fft_rel_err(run_fft(bp, x, direction), ref).max() <= tol(n), (n, direction)
 
 
+# Lengths whose kernel needs fewer registers than its budget: two buffers for each of
+# the blocks that are resident then left 28 KB of L1 (1.23 and 1.25 of the neighbour's
+# time a point; with one buffer 1.03 and 1.05).
+@pytest.mark.parametrize("n,neighbour", [(216, 288), (243, 270)])
+def test_fft_mixed_radix_keeps_the_l1(bp, n, neighbour):
+    total = 1 << 24
+    x = torch.zeros(2 * total, device="cuda")
+    y = torch.empty_like(x)
+
+    def per_point(m):
+        ts = []
+        for _ in range(6):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(20):
+                bp.fft_batched(x, y, m, total // m, -1)
+            e1.record()
+            e1.synchronize()
+            ts.append(e0.elapsed_time(e1))
+        return min(ts) / (total // m * m)
+
+    assert per_point(n) <= 1.14 * per_point(neighbour)
+
+
 def test_fft_mixed_radix_every_length(bp):
     """Every length with a compile-time kernel (all 2^a 3^b 5^c up to 12288
     that are not powers of two), both directions.  Below 1000 points: three
