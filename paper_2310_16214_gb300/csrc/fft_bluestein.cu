@@ -16,7 +16,7 @@
 // iterative radix-2 FFT) and rounded to float32, like the twiddle tables;
 // the data never leaves the GPU.
 //
-// For 32 <= M <= 8192 (and no caller plan) the whole chain is one kernel,
+// For 128 <= M <= 8192 (and no caller plan) the whole chain is one kernel,
 // one signal per M/16 threads: the chirp product is formed as the signal is
 // loaded, the forward M-point transform (the compile-time radix-16 stage
 // schedule) leaves its output in registers, where G multiplies it, and the
@@ -38,7 +38,9 @@ namespace bplg {
 
 namespace {
 
-constexpr int kFusedMinLog = 5, kFusedMaxLog = 13;  // at most 512 threads: 128 registers each
+// n = 33 .. 4096 (shorter lengths have mixed- or prime-radix kernels); at most 512
+// threads: 128 registers each
+constexpr int kFusedMinLog = 7, kFusedMaxLog = 13;
 
 // The fused chain for M = 2^LOGM (radix 16, padded interleaved exchange).
 // Two facts shorten it.  n <= M / 2, so the upper half of the padded input
@@ -48,10 +50,11 @@ constexpr int kFusedMinLog = 5, kFusedMaxLog = 13;  // at most 512 threads: 128 
 // stage reads it: G multiplies in registers and nothing is exchanged between
 // the transforms.  The kernel is bound by the L1 data pipe (per warp and 512
 // points of M, 259 shared wavefronts in four exchanges and 150 for twiddles,
-// chirp and G) and the issue slots together; with the middle exchange and the
-// full halves it took 0.158 ms at n = 1001, 2^24 points, now 0.133; 0.280 ->
-// 0.232 at n = 4095.  Registers: 128, two blocks per SM at M = 2048; capped at
-// 80 or 64 for more blocks it spills (0.160, 0.184 ms).
+// chirp and G) and the issue slots together.  With the middle exchange, the full
+// halves and twiddles r k apart it took, at 2^24 points, 0.164 ms at n = 251, 0.172
+// at 1009 and 0.288 at 4093, now 0.126, 0.131 and 0.231.  Registers: 128, two blocks
+// per SM at M = 2048; capped at 80 or 64 for more blocks it spills (0.160 and 0.184
+// ms where 128 took 0.133).
 template <int LOGM>
 __global__ void __launch_bounds__(512)
     bluestein_fused_kernel(const float2 *__restrict__ x, float2 *__restrict__ X, const float2 *__restrict__ h,
@@ -84,13 +87,11 @@ __global__ void __launch_bounds__(512)
     auto to_out = [&](int pos, float2 val) {
         if (active && pos < n) __stcs(Xs + pos, cmul(val, __ldg(h + pos)));
     };
-    fft_fixed_stages_st<16, LOGM, 1, 0, false, 8>(v, buf2, buf1, j, tw, to_out);
+    fft_fixed_stages_st<16, LOGM, 1, 0, 8>(v, buf2, buf1, j, tw, to_out);
 }
 
 const void *fused_func(int logm) {
     switch (logm) {
-        case 5: return reinterpret_cast<const void *>(&bluestein_fused_kernel<5>);
-        case 6: return reinterpret_cast<const void *>(&bluestein_fused_kernel<6>);
         case 7: return reinterpret_cast<const void *>(&bluestein_fused_kernel<7>);
         case 8: return reinterpret_cast<const void *>(&bluestein_fused_kernel<8>);
         case 9: return reinterpret_cast<const void *>(&bluestein_fused_kernel<9>);

@@ -291,16 +291,13 @@ __device__ __forceinline__ void fft_fixed_stages_reg(float2 (&v)[R], float2 *buf
 }
 
 // All stages, then each output handed with its natural-order position to
-// store(position, value); with SYNC_LAST the block synchronises first (for a
-// store into the exchange buffer that other threads may still be reading).
-// Only registers r < OUT are handed over.
-template <int R, int LOGN, int DIR, int LAYOUT, bool SYNC_LAST = false, int OUT = R, class Store>
+// store(position, value).  Only registers r < OUT are handed over.
+template <int R, int LOGN, int DIR, int LAYOUT, int OUT = R, class Store>
 __device__ __forceinline__ void fft_fixed_stages_st(float2 (&v)[R], float2 *buf2, float *buf1, int j,
                                                     const float2 *__restrict__ tw, Store &store) {
     using O = StageOut<R, LOGN, FftShape<R, LOGN>::NST - 1>;
     fft_fixed_stages_reg<R, LOGN, DIR, LAYOUT, 0>(v, buf2, buf1, j, tw);
     const int ob = O::base(j);
-    if constexpr (SYNC_LAST) __syncthreads();
 #pragma unroll
     for (int r = 0; r < OUT; ++r) store(ob + O::off(r), v[r]);
 }

@@ -1,10 +1,10 @@
 // Uneven-size batches in one launch: problems of different sizes and kinds
 // (the uniform batches of G problems of Section IV-A generalised to mixed
 // sizes) are grouped by (operation, size) into units, largest first, and
-// three persistent kernels -- scan, Stockham FFT, register-level CR/PCR --
-// pull units from one atomic counter each until the work runs out.  The
-// counter reset and the three kernels (on forked branches) are captured once
-// into a CUDA graph, so every run is a single graph launch.
+// three persistent kernels -- scan, Stockham FFT, Wang-Mou solver -- pull
+// units from one atomic counter each until the work runs out.  The counter
+// reset and the three kernels (on forked branches) are captured once into a
+// CUDA graph, so every run is a single graph launch.
 //
 // Units hold up to spb problems of one size; within a unit the layout is
 // the batched kernels' (one signal per T threads), but every problem has its
@@ -87,12 +87,10 @@ __device__ __forceinline__ void scan_unit(const ItemDesc *items, const UnitDesc 
 
 template <typename E>
 __device__ __forceinline__ void scan_unit_dispatch(const ItemDesc *items, const UnitDesc &U, E *warp_tot) {
-    switch (uneven_scan_P(U.logn)) {
-        case 4: scan_unit<E, 4>(items, U, warp_tot); break;
-        case 8: scan_unit<E, 8>(items, U, warp_tot); break;
-        case 16: scan_unit<E, 16>(items, U, warp_tot); break;
-        default: scan_unit<E, 32>(items, U, warp_tot); break;
-    }
+    if (uneven_scan_P(U.logn) == 16)
+        scan_unit<E, 16>(items, U, warp_tot);
+    else
+        scan_unit<E, 32>(items, U, warp_tot);
 }
 
 // five blocks per SM (48 registers; the batch of 3 x 4096 runs 0.0853 ms, with
