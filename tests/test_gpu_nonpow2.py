@@ -313,6 +313,26 @@ def test_fft_bluestein_large_primes_vs_dft(bp, n):
         assert fft_rel_err(run_fft(bp, x, direction), oracle.dft(x, direction)).max() <= tol(n), (n, direction)
 
 
+# the other inner lengths of the fused kernel (M = 128, 512, 1024), and blocks of many
+# signals: several blocks, the last one not full
+@pytest.mark.parametrize("n,batch", [(37, 70), (61, 33), (251, 19), (509, 9), (1009, 3)])
+def test_fft_bluestein_blocks_of_signals(bp, n, batch):
+    x = si.fft_c64(batch, n, stream=2600 + n)
+    for direction in (-1, 1):
+        assert fft_rel_err(run_fft(bp, x, direction), oracle.dft(x, direction)).max() <= tol(n), (n, direction)
+
+
+# in place, through the fused kernel and through the five kernels of M > 8192
+@pytest.mark.parametrize("n,batch", [(37, 70), (1009, 9), (4093, 3), (4099, 2), (8191, 2)])
+def test_fft_bluestein_in_place(bp, n, batch):
+    x = si.fft_c64(batch, n, stream=2650 + n)
+    buf = c64_to_dev(x)
+    bp.fft_batched(buf, buf, n, batch, -1)
+    assert np.array_equal(c64_from_dev(buf).reshape(batch, n), run_fft(bp, x, -1))
+    bp.fft_batched(buf, buf, n, batch, 1)
+    assert fft_rel_err(c64_from_dev(buf).reshape(batch, n) / n, x.astype(np.complex128)).max() <= 2 * tol(n)
+
+
 # prime radices 7 .. 31: every radix first, in the middle and last, one stage to
 # five, one signal a block and many (the last block not full), the longest
 # length; in place too.  Above 2100 points against numpy's float64 FFT.
