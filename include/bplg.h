@@ -181,7 +181,9 @@ int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64
  *          (see n1_log in the plan) through a scratch buffer of n * batch
  *          complex values that the library allocates on first use per device
  *          and stream and grows when needed (a growth waits for the stream);
- *          in may equal out.
+ *          in may equal out.  Its first call with an n also makes a table of
+ *          n / 16 complex values (8 MB at 2^24), and its first call with a
+ *          row length N2 one of 16 N2 (2 MB at 2^14), both kept.
  *          A length n = 2^a 3^b 5^c up to 12288 that is not a power of two
  *          (and no plan) runs a mixed-radix Stockham kernel compiled for
  *          that length: stages of radix 2, 3, 4, 5, 6, 8, 9, 10, 12, 15 or

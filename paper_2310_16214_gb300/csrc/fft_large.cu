@@ -31,8 +31,8 @@
 // Thread j of a column holds the outputs k1 = j + r T, T = N1 / 16, r < 16, so
 //     W_n^(k1 n2) = W_n^(j n2) W_(16 N2)^(r n2),
 // a product of two float64-generated, once-rounded factors: W_n^m, m < n / 16
-// (a table per n), one load for a thread's 16 outputs; and the stage table
-// [r][n2] of 16 N2 entries (one per N2 and device), read with the column n2
+// (a table per n and device), one load for a thread's 16 outputs; and the stage
+// table [r][n2] of 16 N2 entries (one per N2 and device), read with the column n2
 // across the lanes.  (W_n^(k1 n2 mod 4096) W_n^(4096 (k1 n2 div 4096)) took
 // every output two loads whose lanes lay k1 entries apart, three quarters of
 // the column kernel's L1 work: 0.139 -> 0.127 ms at 2^20 points, 16 signals.)
@@ -172,34 +172,35 @@ __global__ void large_root_kernel(float2 *t, int logn, int64_t count) {
     t[m] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
 }
 
-// t[16 N2 + r N2 + n2] = W_(16 N2)^(r n2) for every N2 of a row pass
-__global__ void large_stage_kernel(float2 *t, int64_t count) {
+// t[r N2 + n2] = W_(16 N2)^(r n2), r < 16, N2 = 2^logn2
+__global__ void large_stage_kernel(float2 *t, int logn2) {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= count || i < (int64_t(16) << kLargeMinPassLog)) return;
-    const int logm = 63 - __clzll(static_cast<unsigned long long>(i));  // 16 N2 = 2^logm
-    const int64_t e = i - (int64_t(1) << logm), n2 = int64_t(1) << (logm - 4);
+    if (i >= int64_t(16) << logn2) return;
+    const int64_t r = i >> logn2, n2 = i & ((int64_t(1) << logn2) - 1);
     double sn, cs;
-    sincospi(-2.0 * static_cast<double>((e / n2) * (e % n2)) / static_cast<double>(int64_t(1) << logm), &sn, &cs);
+    sincospi(-2.0 * static_cast<double>(r * n2) / static_cast<double>(int64_t(16) << logn2), &sn, &cs);
     t[i] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
 }
 
 std::mutex g_mu;
-std::map<std::pair<int, int>, float2 *> g_root;  // (device, log n) -> W_n^m; (device, 0) -> the stage tables
+// (device, log n) -> W_n^m; (device, -log N2) -> the stage table of a row length
+std::map<std::pair<int, int>, float2 *> g_tables;
 // (device, stream, tag) -> (buffer, bytes)
 std::map<std::tuple<int, cudaStream_t, int>, std::pair<void *, size_t>> g_scratch;
 
-// the table of W_n^m, m < n / 16, or (logn 0) the stage tables
-int large_table(int logn, const float2 **out) {
+// the table of W_n^m, m < n / 16 (which = log n > 0), or the stage table of rows of
+// N2 points (which = -log N2)
+int large_table(int which, const float2 **out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
     std::lock_guard<std::mutex> lock(g_mu);
-    auto it = g_root.find({dev, logn});
-    if (it != g_root.end()) {
+    auto it = g_tables.find({dev, which});
+    if (it != g_tables.end()) {
         *out = it->second;
         return BPLG_OK;
     }
-    const int64_t count = logn > 0 ? int64_t(1) << (logn - 4) : int64_t(32) << kLargeMaxPassLog;
+    const int64_t count = which > 0 ? int64_t(1) << (which - 4) : int64_t(16) << -which;
     float2 *p = nullptr;
     e = cudaMalloc(&p, sizeof(float2) * static_cast<size_t>(count));
     if (e != cudaSuccess) return cuda_error(e, "large twiddle cudaMalloc");
@@ -210,10 +211,10 @@ int large_table(int logn, const float2 **out) {
         return cuda_error(e, "large twiddle stream");
     }
     const unsigned blocks = static_cast<unsigned>((count + 255) / 256);
-    if (logn > 0)
-        large_root_kernel<<<blocks, 256, 0, st>>>(p, logn, count);
+    if (which > 0)
+        large_root_kernel<<<blocks, 256, 0, st>>>(p, which, count);
     else
-        large_stage_kernel<<<blocks, 256, 0, st>>>(p, count);
+        large_stage_kernel<<<blocks, 256, 0, st>>>(p, -which);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     cudaStreamDestroy(st);
@@ -221,7 +222,7 @@ int large_table(int logn, const float2 **out) {
         cudaFree(p);
         return cuda_error(e, "large twiddle generation");
     }
-    g_root[{dev, logn}] = p;
+    g_tables[{dev, which}] = p;
     *out = p;
     return BPLG_OK;
 }
@@ -348,9 +349,8 @@ int fft_large_launch(const bplg_plan &p, const void *in, void *out, int64_t n, i
     int logn = ilog2(n);
     const float2 *root = nullptr, *stage = nullptr;
     rc = large_table(logn, &root);
-    if (rc == BPLG_OK) rc = large_table(0, &stage);
+    if (rc == BPLG_OK) rc = large_table(p.n1_log - logn, &stage);
     if (rc != BPLG_OK) return rc;
-    stage += n >> (p.n1_log - 4);  // the block of 16 N2
     void *y = nullptr;
     rc = stream_scratch(kScratchLargeFft, static_cast<size_t>(n) * static_cast<size_t>(batch) * sizeof(float2), s, &y);
     if (rc != BPLG_OK) return rc;

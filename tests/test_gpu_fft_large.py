@@ -4,6 +4,10 @@ order) against the float64 oracle: relative L2 error per signal
 <= 1e-5 * log2 N, forward and inverse, every plan at 2^15, the default plan
 up to 2^22, in place, closed forms."""
 import math
+import os
+import pathlib
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -15,6 +19,8 @@ from tests.gpu_util import c64_from_dev, c64_to_dev, fft_rel_err
 pytestmark = pytest.mark.gpu
 
 torch = pytest.importorskip("torch")
+
+ROOT = pathlib.Path(__file__).resolve().parent.parent
 
 
 @pytest.fixture(scope="module")
@@ -62,6 +68,26 @@ def test_every_row_count_per_block(bp, row_log):
         for d in (-1, 1):
             assert fft_rel_err(run(bp, z, d, p), ref[d]).max() <= 1e-5 * logn, (p, d)
     assert bp.device_status() == 0
+
+
+def test_device_memory_of_a_first_call(bp):
+    """One transform of 2^16 points makes its own two tables (64 KB) and its
+    scratch (512 KB), not those of every row length (4 MB)."""
+    code = """
+import torch, paper_2310_16214_gb300 as bp
+x = torch.zeros(2 << 16, device="cuda")
+y = torch.empty_like(x)
+bp.fft_batched(x, y, 4096, 1, -1)  # the shared table
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+bp.fft_batched(x, y, 1 << 16, 1, -1)
+torch.cuda.synchronize()
+print(free - torch.cuda.mem_get_info()[0])
+"""
+    env = dict(os.environ, CUDA_MODULE_LOADING="EAGER")  # no kernel is loaded in between
+    r = subprocess.run([sys.executable, "-c", code], env=env, cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    assert int(r.stdout) <= 2 << 20
 
 
 @pytest.mark.parametrize("logn", [16, 18, 20, 22])
