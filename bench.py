@@ -1165,11 +1165,11 @@ def largefft_report(args):
 
 
 def nonpow2_report(args):
-    """Lengths that are not powers of two, 2^24 elements per case: the padded
-    scan (int32) and Wang-Mou solve on the next power of two against the
-    power-of-two length just below, and FFTs against cuFFT (mixed radix for
-    2^a 3^b 5^c up to 12288, Bluestein otherwise; cuFFT runs such lengths
-    with its own mixed-radix or Bluestein kernels).  Every
+    """Lengths that are not powers of two, 2^24 elements per case: the
+    scan (int32) and the Wang-Mou solve against the power-of-two length
+    just below, and FFTs against cuFFT (mixed radix for 2^a 3^b 5^c up to
+    12288, prime radices 7 to 31 up to 12288, Bluestein otherwise; cuFFT runs
+    such lengths with its own mixed-radix or Bluestein kernels).  Every
     row reports the time, Gelem/s and the fraction of the measured copy
     bandwidth for the algorithmic bytes (scan 8, tridiag 20, FFT 16 per
     element)."""

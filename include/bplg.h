@@ -166,7 +166,11 @@ typedef struct {
  *          any other n runs a plan of the next power of two n' (plan->n ==
  *          n'; plan NULL: one chosen for n and batch), the rows read as if
  *          padded with zeros to n' (rows stay n apart, nothing outside a row
- *          is read or written).
+ *          is read or written).  When n is not a multiple of 4 the float32
+ *          sums of a row may be formed in an order that depends on where the
+ *          row starts within its 16 bytes, so equal rows at different places
+ *          of a batch can differ in their last bits (a call repeated on the
+ *          same data does not).
  * Errors: INVALID_ARG, UNSUPPORTED_SIZE, INVALID_PLAN, CUDA. */
 int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64_t batch,
                       const bplg_plan *plan, void *stream);
@@ -186,18 +190,18 @@ int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64
  *          row length N2 one of 16 N2 (2 MB at 2^14), both kept.
  *          A length n = 2^a 3^b 5^c up to 12288 that is not a power of two
  *          (and no plan) runs a mixed-radix Stockham kernel compiled for
- *          that length: stages of radix 2, 3, 4, 5, 6, 8, 9, 10, 12, 15 or
- *          16, the block's signals in shared memory, the stage twiddles
- *          from a per-n table made on the first call with that n
- *          (float64 on the host, rounded to float32, uploaded
- *          synchronously).
+ *          that length: stages of radix 2, 3, 4, 5, 6, 8, 9, 10, 12, 15,
+ *          16, 18, 20, 24 or 25, the block's signals in shared memory, the
+ *          stage twiddles from a per-n table made on the first call with
+ *          that n (float64 on the host, rounded to float32, on the device
+ *          before the first kernel).
  *          Any other length up to 12288 whose prime factors are at most 31
  *          (and no plan) runs the same stages planned at run time, with prime
  *          radices 7 to 31, and a table made the same way.
  *          Any other length that is not a power of two runs Bluestein's
  *          chirp identity: X_k = h_k sum_j (x_j h_j) conj(h_{k-j}) with
  *          h_m = exp(dir pi i m^2 / n), a cyclic convolution of length
- *          M = next power of two >= 2n - 1.  With no plan and 32 <= M <=
+ *          M = next power of two >= 2n - 1.  With no plan and 128 <= M <=
  *          8192 it is one fused kernel; otherwise (or with a plan, which
  *          must be made for M) two M-point FFTs and three elementwise
  *          kernels through a scratch of M * batch complex values per device
@@ -286,7 +290,11 @@ int bplg_fft_batched_noalloc(const void *in, void *out, int64_t n, int64_t batch
  *           written.  With plan NULL most such n above 256, in all but small
  *           batches, run a persistent form of the solver with its own tiling,
  *           fed by bulk copies in whole 16-byte units: up to three elements on
- *           either side of a row may be read, none outside the arrays.
+ *           either side of a row may be read, none outside the arrays.  When
+ *           n is not a multiple of 4 that tiling shifts with the place of the
+ *           row within its 16 bytes: equal systems at different places of a
+ *           batch can then differ in their last bits (a call repeated on the
+ *           same data does not), and n and batch choose between the forms.
  * No pivoting: the systems must be safe for elimination without pivoting
  * (e.g. strictly diagonally dominant).  Pivots are inverted with the fast
  * float32 reciprocal (__fdividef(1, x)), which gives 0 for |x| > 2^126, so

@@ -320,7 +320,7 @@ bool tridiag_wm_tma_applies(int64_t n, int64_t batch) {
 
 int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const float *d, float *x, int64_t n,
                           int64_t batch, cudaStream_t s) {
-    const int max_shift = n % 4 == 0 ? 0 : (n % 2 == 0 ? 2 : 3);  // rows before the first in its 16 bytes
+    const int max_shift = n % 4 == 0 ? 0 : (n % 2 == 0 ? 2 : 3);  // elements before a row in its first 16 bytes
     const auto threads = [&](int P) { return static_cast<int>((n + max_shift + 32 * P - 1) / (32 * P) * 32); };
     // P = 12, or 20 where that leaves fewer threads idle: one warp instead of two
     // (n = 385 .. 640), and above 2048 (n = 2500 0.0665 -> 0.0613 ms, 3500 0.0734 -> 0.0643,

@@ -291,8 +291,8 @@ def run_fft(bp, x, direction, plan=None, guard=16):
     return o[:2 * batch * n].view(np.complex64).reshape(batch, n)
 
 
-# lengths with a prime factor above 5: Bluestein (fused kernel for M = 32 ..
-# 8192, i.e. n = 17 .. 4096; three launches below and above)
+# lengths with a prime factor above 5 (these run prime radices now; Bluestein's
+# lengths, with a prime factor above 31, follow)
 @pytest.mark.parametrize("n", [7, 14, 77, 1001, 4095])
 def test_fft_bluestein_vs_dft(bp, n):
     batch = 6 if n <= 1001 else 2
@@ -356,7 +356,7 @@ def test_fft_prime_radices(bp, n, batch):
 
 
 # 2^a 3^b 5^c (not a power of two, at most 12288): the mixed-radix Stockham
-# kernels (one per length, radices 2 .. 16); small lengths several signals a
+# kernels (one per length, radices 2 .. 25); small lengths several signals a
 # block (ragged last block)
 @pytest.mark.parametrize("n", [3, 5, 6, 9, 10, 12, 15, 20, 25, 27, 45, 60, 81, 100, 120, 125, 243, 360, 375, 625,
                                1000, 1215, 1536, 2187, 3000])
