@@ -65,16 +65,27 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 
 // Wait for phase `parity` of `bar` with a time limit; false (and the device
 // error word set) if the limit passed.
-__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity,
+                                                  long long limit = kWaitLimitCycles) {
     if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (!mbar_try_wait(bar, parity)) {
-        if (clock64() - t0 > kWaitLimitCycles) {
+        if (clock64() - t0 > limit) {
             atomicExch(&g_device_error, kErrWaitTimeout);
             return false;
         }
     }
     return true;
+}
+
+// The same by every thread of a block with one phase in flight, which leaves when
+// the vote on it fails.  The leader waits twice as long, so when the vote fails the
+// copies have been waited for again and have landed, or that has run out too: the
+// shared memory may belong to another block afterwards.  (A wait after the vote
+// does the same, but its code in the loop cost the bulk-copy tridiagonal solver 4 us
+// of 60 at n = 3000.)
+__device__ __forceinline__ bool mbar_wait_block(uint64_t *bar, uint32_t parity, bool leader) {
+    return mbar_wait_bounded(bar, parity, leader ? 2 * kWaitLimitCycles : kWaitLimitCycles);
 }
 
 }  // namespace bplg

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     __syncthreads();
     uint32_t parity = 0;
     for (int64_t sys = blockIdx.x; sys < batch; sys += gridDim.x, parity ^= 1u) {
-        const bool ok = mbar_wait_bounded(&full, parity);
+        const bool ok = mbar_wait_block(&full, parity, t == 0);
         float a[P], b[P], c[P], d[P];
         const float4 *s4 = reinterpret_cast<const float4 *>(slot + t * P);
 #pragma unroll
@@ -189,13 +189,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
             d[4 * q] = vd.x; d[4 * q + 1] = vd.y; d[4 * q + 2] = vd.z; d[4 * q + 3] = vd.w;
         }
         // the slot is read (and the exchange buffers of the last system too)
-        if (!__syncthreads_and(ok)) {
-            // a wait ran out: the block leaves once its copies, one phase at most,
-            // have landed (or the second wait for them has run out too), because the
-            // slot may belong to another block afterwards
-            if (t == 0) mbar_wait_bounded(&full, parity);
-            return;
-        }
+        if (!__syncthreads_and(ok)) return;  // a wait ran out; thread 0 has waited again
         if (t == 0 && sys + gridDim.x < batch) {
             fence_proxy_async();
             issue(sys + gridDim.x);

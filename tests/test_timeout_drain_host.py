@@ -42,4 +42,14 @@ def test_block_drains_its_copies_before_leaving(name):
     for m in tests:
         body = _block(text, m.end())
         if "return" in body:
-            assert "mbar_wait_bounded" in body[:body.index("return")], "%s: %s" % (name, body)
+            # either it waits again before it leaves, or the wait voted on is the one
+            # whose leader waits twice as long
+            again = "mbar_wait_bounded" in body[:body.index("return")]
+            waits = re.findall(r"mbar_wait_(?:bounded|block)\(", text[:m.start()] + m.group())
+            assert again or waits[-1] == "mbar_wait_block(", "%s: %s" % (name, body)
+
+
+def test_the_leader_waits_longer():
+    text = (CSRC / "tma.cuh").read_text()
+    assert re.search(r"bool mbar_wait_block\([^)]*bool leader\) \{\s*return mbar_wait_bounded\(bar, parity, "
+                     r"leader \? 2 \* kWaitLimitCycles : kWaitLimitCycles\);", text)
