@@ -295,21 +295,24 @@ int tridiag_wm_device_status(int *flag, bool reset) {
 
 // Which calls take it: lengths above 256 whose padded form wastes threads or has
 // rows off 16-byte boundaries, unless
-//   - a multiple of 4 above three quarters of the power of two, up to 2048: of the
-//     padded form's threads (P = 8) nearly all are busy, and without a slot in shared
-//     memory more of its blocks fit an SM (2^24 unknowns, padded / bulk copies: n = 400
-//     60 / 66 us, 800 64 / 76, 1600 62 / 72, 2000 58 / 67, but 768 66 / 61, 1500 66 / 59,
-//     4000 74 / 74); up to 256 a block here is one warp with half of its lanes idle;
+//   - a multiple of 4 above three quarters of the power of two, up to 2048, other than
+//     1684 .. 1920 (five nearly full warps of P = 12): of the padded form's threads (P =
+//     8) nearly all are busy, and without a slot in shared memory more of its blocks fit
+//     an SM (2^24 unknowns, padded / bulk copies: n = 392 59 / 64 us, 500 52 / 55, 800 63 /
+//     70, 1544 63 / 66, 2000 57 / 60, but 380 60 / 59, 764 65 / 60, 1532 63 / 56, 1800 60 /
+//     58, 4032 72 / 69); up to 256 a block here is one warp with half of its lanes idle;
 //   - few systems, which take as long as one, the longer the more equations a thread
-//     has (device time, padded / bulk copies: 76 systems of n = 300 2.5 / 3.2 us, 491 2.6
-//     / 3.7, 1100 3.2 / 3.7, 3600 4.6 / 5.4, but 1025 4.4 / 3.7, 6500 6.8 / 6.5; the two
-//     meet at 2400 systems of 300, 900 of 600, 600 of 1500, 300 of 2200, 300 of 641, 150
-//     of 901).
+//     has (device time, padded / bulk copies: 76 systems of n = 300 2.5 / 3.1 us, 491 2.7
+//     / 3.6, 1100 3.2 / 3.6, 3600 4.7 / 5.4, but 1025 4.4 / 3.6, 6500 6.8 / 6.5; the two
+//     meet at 1800 systems of 300, 900 of 600, 350 of 1100, 450 of 1500, 300 of 2200 and
+//     641, 150 of 901).
 bool tridiag_wm_tma_applies(int64_t n, int64_t batch) {
     if (is_pow2(n) || n <= 256 || n > (int64_t(1) << kTridiagMaxLog)) return false;
-    const int64_t few = n % 4 == 0 ? (n <= 384 ? 2432 : (n <= 2048 ? 608 : (n <= 4096 ? 152 : 0)))
-                                   : (n <= 640 ? 304 : (n <= 900 ? 152 : 0));
-    return batch > few && (n % 4 != 0 || n > 2048 || 4 * n <= 3 * next_pow2(n));
+    const bool aligned = n % 4 == 0;
+    const int64_t few = aligned ? (n <= 384 ? 1824 : (n <= 1024 ? 608 : (n <= 2048 ? 304 : (n <= 4096 ? 152 : 0))))
+                                : (n <= 640 ? 304 : (n <= 900 ? 152 : 0));
+    const bool full = aligned && n < 2048 && 4 * n > 3 * next_pow2(n) && (n <= 1680 || n > 1920);
+    return batch > few && !full;
 }
 
 int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const float *d, float *x, int64_t n,

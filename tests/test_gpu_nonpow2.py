@@ -217,10 +217,11 @@ def test_tridiag_rows_off_alignment(bp, n, batch):
 
 # The bulk-copy solver and the padded one take turns over length and batch: both
 # sides of each line, every shape of the bulk-copy solver in batches large enough for it.
-@pytest.mark.parametrize("n,batch", [(380, 2433), (384, 2432), (384, 2433), (388, 700), (385, 304), (385, 305), (637, 310),
+@pytest.mark.parametrize("n,batch", [(380, 1825), (384, 1824), (384, 1825), (388, 700), (385, 304), (385, 305), (637, 310),
                                      (640, 609), (641, 152), (641, 153), (768, 608), (768, 609), (772, 700), (900, 160),
-                                     (901, 2), (1500, 609), (1536, 609), (1540, 620), (2044, 609), (2052, 152), (2052, 153),
-                                     (4092, 153), (4100, 1)])
+                                     (901, 2), (1500, 304), (1500, 305), (1536, 609), (1540, 620), (1680, 305), (1684, 305),
+                                     (1920, 305), (1924, 305), (2044, 609), (2052, 152), (2052, 153), (4092, 153),
+                                     (4100, 1)])
 def test_tridiag_ragged_lines(bp, n, batch):
     a, b, c, d, _ = si.tridiag_f32(batch, n, stream=1900 + n)
     a[:, 0] = np.nan  # never read
