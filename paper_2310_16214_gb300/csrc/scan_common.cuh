@@ -21,14 +21,12 @@ namespace bplg {
 // RUNS: P consecutive elements a thread all the same, one prefix for them.
 template <int P, bool RUNS = false>
 struct ScanRows {
-    static constexpr int W = P < 4 ? P : 4;       // elements of one access
-    static constexpr int V = RUNS ? P : W;        // adjacent elements that share a prefix
-    static constexpr int ROWS = P / V;
+    static constexpr int W = P < 4 ? P : 4;  // elements of one access
     static constexpr int GROUPS = P / W;
     // first element of thread t's access q in its problem of tps threads
     __device__ __forceinline__ static int pos(int t, int tps, int q) {
-        if (ROWS == 1) return t * P + q * W;
-        return tps >= 32 ? (t >> 5) * (32 * P) + q * (32 * V) + (t & 31) * V : q * (tps * V) + t * V;
+        if (RUNS || GROUPS == 1) return t * P + q * W;
+        return tps >= 32 ? (t >> 5) * (32 * P) + q * (32 * W) + (t & 31) * W : q * (tps * W) + t * W;
     }
 };
 
@@ -41,18 +39,47 @@ __device__ __forceinline__ void scan_problem(E (&v)[P], int tps, int wl, E *warp
     const int lane = threadIdx.x & 31;
     const int width = tps < 32 ? tps : 32;
     const int lane_in_seg = lane & (width - 1);
-    E add[S::ROWS];  // what each row of the thread gets from the rows and lanes before it
-    E off = E(0);    // in the last lane of a segment finally the segment's total
+    // Every four elements (or fewer) have a prefix of their own and get what is before
+    // them in one addition.  (A serial prefix over all of a run of 16 rounded on, at n =
+    // 260 to a relative error of 9.5e-8 where this has 7.8e-8.)
+    constexpr bool kRuns = RUNS && S::GROUPS > 1;
+    E add[S::GROUPS];  // what each four get from those before them
+    E off = E(0);      // in the last lane of a segment finally the segment's total
 #pragma unroll
-    for (int q = 0; q < S::ROWS; ++q)
+    for (int q = 0; q < S::GROUPS; ++q) {
+        E *g = v + S::W * q;
+        if constexpr (kRuns) {  // sums in pairs
+            const E cd = g[2] + g[3];
+            g[1] += g[0];
+            g[2] += g[1];
+            g[3] = g[1] + cd;
+        } else {
 #pragma unroll
-        for (int i = 1; i < S::V; ++i) v[S::V * q + i] += v[S::V * q + i - 1];
+            for (int i = 1; i < S::W; ++i) g[i] += g[i - 1];
+        }
+    }
+    if constexpr (kRuns) {
+        E run = E(0);  // the run's total after the loop
 #pragma unroll
-    for (int q = 0; q < S::ROWS; ++q) {
-        const E incl = seg_scan<PATTERN>(v[S::V * q + S::V - 1], lane_in_seg, width);
+        for (int q = 0; q < S::GROUPS; q += 2) {
+            const E g0 = v[S::W * q + S::W - 1], g1 = v[S::W * (q + 1) + S::W - 1];
+            add[q] = run;
+            add[q + 1] = run + g0;
+            run += g0 + g1;
+        }
+        const E incl = seg_scan<PATTERN>(run, lane_in_seg, width);
         const E excl = __shfl_up_sync(kFullMask, incl, 1, width);
-        add[q] = off + (lane_in_seg == 0 ? E(0) : excl);
-        off += q + 1 < S::ROWS ? __shfl_sync(kFullMask, incl, width - 1, width) : incl;
+#pragma unroll
+        for (int q = 0; q < S::GROUPS; ++q) add[q] += lane_in_seg == 0 ? E(0) : excl;
+        off = incl;
+    } else {
+#pragma unroll
+        for (int q = 0; q < S::GROUPS; ++q) {
+            const E incl = seg_scan<PATTERN>(v[S::W * q + S::W - 1], lane_in_seg, width);
+            const E excl = __shfl_up_sync(kFullMask, incl, 1, width);
+            add[q] = off + (lane_in_seg == 0 ? E(0) : excl);
+            off += q + 1 < S::GROUPS ? __shfl_sync(kFullMask, incl, width - 1, width) : incl;
+        }
     }
     if (tps > 32) {
         const int warp = threadIdx.x >> 5;
@@ -64,12 +91,12 @@ __device__ __forceinline__ void scan_problem(E (&v)[P], int tps, int wl, E *warp
         E before = __shfl_sync(kFullMask, w, wl > 0 ? wl - 1 : 0);
         if (wl == 0) before = E(0);
 #pragma unroll
-        for (int q = 0; q < S::ROWS; ++q) add[q] += before;
+        for (int q = 0; q < S::GROUPS; ++q) add[q] += before;
     }
 #pragma unroll
-    for (int q = 0; q < S::ROWS; ++q)
+    for (int q = 0; q < S::GROUPS; ++q)
 #pragma unroll
-        for (int i = 0; i < S::V; ++i) v[S::V * q + i] += add[q];
+        for (int i = 0; i < S::W; ++i) v[S::W * q + i] += add[q];
 }
 
 // One access of a thread: V elements at p, aligned to V elements.

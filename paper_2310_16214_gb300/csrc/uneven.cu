@@ -71,18 +71,18 @@ __device__ __forceinline__ void scan_unit(const ItemDesc *items, const UnitDesc 
     }
     E v[P];
 #pragma unroll
-    for (int q = 0; q < S::ROWS; ++q) {
+    for (int q = 0; q < S::GROUPS; ++q) {
         if (active) {
-            load_row<E, S::V>(in + S::pos(t, T, q), v + S::V * q);
+            load_row<E, S::W>(in + S::pos(t, T, q), v + S::W * q);
         } else {
 #pragma unroll
-            for (int i = 0; i < S::V; ++i) v[S::V * q + i] = E(0);
+            for (int i = 0; i < S::W; ++i) v[S::W * q + i] = E(0);
         }
     }
     scan_problem<E, P, 0>(v, T, (tid >> 5) & ((T >> 5) - 1), warp_tot);
     if (!active) return;
 #pragma unroll
-    for (int q = 0; q < S::ROWS; ++q) store_row<E, S::V>(out + S::pos(t, T, q), v + S::V * q);
+    for (int q = 0; q < S::GROUPS; ++q) store_row<E, S::W>(out + S::pos(t, T, q), v + S::W * q);
 }
 
 template <typename E>
