@@ -207,7 +207,9 @@ int bplg_tridiag_batched(const float *a, const float *b, const float *c, const f
         return tridiag_wm_tma_launch(a, b, c, d, x, n, batch, static_cast<cudaStream_t>(stream));
     const int op = np != n || (plan && plan->op == BPLG_OP_TRIDIAG_WM) ? BPLG_OP_TRIDIAG_WM : BPLG_OP_TRIDIAG;
     OnlineTicket tk;
-    int rc = resolve_plan(op, BPLG_F32, np, batch, plan, &p, np == n ? &tk : nullptr);
+    int rc = BPLG_OK;
+    if (plan || !tridiag_wm_padded_plan(n, batch, &p))
+        rc = resolve_plan(op, BPLG_F32, np, batch, plan, &p, np == n ? &tk : nullptr);
     if (rc != BPLG_OK) return rc;
     p.n = static_cast<int32_t>(np);
     const cudaStream_t s = static_cast<cudaStream_t>(stream);

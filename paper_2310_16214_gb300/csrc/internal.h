@@ -86,6 +86,7 @@ int tridiag_wm_launch(const bplg_plan &p, const float *a, const float *b, const 
                       int64_t n, int64_t batch, cudaStream_t s);
 // its persistent bulk-copy form for lengths that are not powers of two
 bool tridiag_wm_tma_applies(int64_t n, int64_t batch);
+bool tridiag_wm_padded_plan(int64_t n, int64_t batch, bplg_plan *p);  // false: another decides
 int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const float *d, float *x, int64_t n,
                           int64_t batch, cudaStream_t s);
 int tridiag_refined_launch(const bplg_plan &p, const float *a, const float *b, const float *c,

@@ -298,9 +298,10 @@ int tridiag_wm_device_status(int *flag, bool reset) {
 //   - a multiple of 4 above three quarters of the power of two, up to 2048, other than
 //     1684 .. 1920 (five nearly full warps of P = 12): of the padded form's threads (P =
 //     8) nearly all are busy, and without a slot in shared memory more of its blocks fit
-//     an SM (2^24 unknowns, padded / bulk copies: n = 392 59 / 64 us, 500 52 / 55, 800 63 /
-//     70, 1544 63 / 66, 2000 57 / 60, but 380 60 / 59, 764 65 / 60, 1532 63 / 56, 1800 60 /
-//     58, 4032 72 / 69); up to 256 a block here is one warp with half of its lanes idle;
+//     an SM (2^24 unknowns, cost model's plan padded / bulk copies: n = 392 59 / 64 us,
+//     500 52 / 55, 800 63 / 70, 1544 63 / 66, 2000 57 / 60, but 380 60 / 59, 764 65 / 60,
+//     1532 63 / 56, 1800 60 / 58, 4032 72 / 69); up to 256 a block here is one warp with
+//     half of its lanes idle;
 //   - few systems, which take as long as one, the longer the more equations a thread
 //     has (device time, padded / bulk copies: 76 systems of n = 300 2.5 / 3.1 us, 491 2.7
 //     / 3.6, 1100 3.2 / 3.6, 3600 4.7 / 5.4, but 1025 4.4 / 3.6, 6500 6.8 / 6.5; the two
@@ -313,6 +314,24 @@ bool tridiag_wm_tma_applies(int64_t n, int64_t batch) {
                                 : (n <= 640 ? 304 : (n <= 900 ? 152 : 0));
     const bool full = aligned && n < 2048 && 4 * n > 3 * next_pow2(n) && (n <= 1680 || n > 1920);
     return batch > few && !full;
+}
+
+// The padded kernel's plan for those calls above 256 whose power of two is at most 1024,
+// without a plan tuned for it: P = 16, one system a block.  (The cost model's plan, P
+// = 8, suits whole systems: n = 400 59.8 us at 2^24 unknowns, this one 53.8; 800 63.9,
+// 55.6; and its sums, of twice the threads, are further from float64, 6.66e-8 against
+// 6.41e-8.)
+bool tridiag_wm_padded_plan(int64_t n, int64_t batch, bplg_plan *p) {
+    const int64_t np = next_pow2(n);
+    if (np == n || np < 512 || np > 1024 || cache_lookup(BPLG_OP_TRIDIAG_WM, BPLG_F32, np, batch, p)) return false;
+    *p = {};
+    p->op = BPLG_OP_TRIDIAG_WM;
+    p->P = 16;
+    p->spb = 1;
+    p->radix = 2;
+    p->shuffle = 1;
+    plan_finalize(p, BPLG_F32, np);
+    return true;
 }
 
 int tridiag_wm_tma_launch(const float *a, const float *b, const float *c, const float *d, float *x, int64_t n,
