@@ -186,8 +186,9 @@ int bplg_scan_batched(int32_t dtype, const void *in, void *out, int64_t n, int64
  *          complex values that the library allocates on first use per device
  *          and stream and grows when needed (a growth waits for the stream);
  *          in may equal out.  Its first call with an n also makes a table of
- *          n / 16 complex values (8 MB at 2^24), and its first call with a
- *          row length N2 one of 16 N2 (2 MB at 2^14), both kept.
+ *          n / 16 complex values (8 MB at 2^24) and one of 16 N2 for each row
+ *          length N2 its plans can have that has none yet (4 MB for all of
+ *          2^6 .. 2^14, 250 KB at n = 2^16), all kept.
  *          A length n = 2^a 3^b 5^c up to 12288 that is not a power of two
  *          (and no plan) runs a mixed-radix Stockham kernel compiled for
  *          that length: stages of radix 2, 3, 4, 5, 6, 8, 9, 10, 12, 15,

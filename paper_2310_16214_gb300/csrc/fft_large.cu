@@ -188,42 +188,46 @@ std::map<std::pair<int, int>, float2 *> g_tables;
 // (device, stream, tag) -> (buffer, bytes)
 std::map<std::tuple<int, cudaStream_t, int>, std::pair<void *, size_t>> g_scratch;
 
-// the table of W_n^m, m < n / 16 (which = log n > 0), or the stage table of rows of
-// N2 points (which = -log N2)
-int large_table(int which, const float2 **out) {
+// The table of W_n^m, m < n / 16, and the stage table of rows of 2^logn2 points.  The
+// first call with an n makes its own and those of every row length a plan of n can
+// have, so that a call under capture needs no more than a call with that n before it.
+int large_tables(int logn, int logn2, const float2 **root, const float2 **stage) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return cuda_error(e, "cudaGetDevice");
     std::lock_guard<std::mutex> lock(g_mu);
-    auto it = g_tables.find({dev, which});
-    if (it != g_tables.end()) {
-        *out = it->second;
-        return BPLG_OK;
+    if (g_tables.find({dev, logn}) == g_tables.end()) {
+        cudaStream_t st;
+        e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e != cudaSuccess) return cuda_error(e, "large twiddle stream");
+        std::map<std::pair<int, int>, float2 *> made;
+        auto make = [&](int which, int64_t count) {
+            if (e != cudaSuccess || g_tables.find({dev, which}) != g_tables.end()) return;
+            float2 *p = nullptr;
+            e = cudaMalloc(&p, sizeof(float2) * static_cast<size_t>(count));
+            if (e != cudaSuccess) return;
+            made[{dev, which}] = p;
+            const unsigned blocks = static_cast<unsigned>((count + 255) / 256);
+            if (which > 0)
+                large_root_kernel<<<blocks, 256, 0, st>>>(p, which, count);
+            else
+                large_stage_kernel<<<blocks, 256, 0, st>>>(p, -which);
+            e = cudaGetLastError();
+        };
+        make(logn, int64_t(1) << (logn - 4));
+        for (int l = kLargeMinPassLog; l <= kLargeMaxPassLog; ++l)
+            if (logn - l >= kLargeMinPassLog && logn - l <= kLargeMaxPassLog) make(-l, int64_t(16) << l);
+        const cudaError_t done = cudaStreamSynchronize(st);
+        cudaStreamDestroy(st);
+        if (e == cudaSuccess) e = done;
+        if (e != cudaSuccess) {
+            for (auto &t : made) cudaFree(t.second);
+            return cuda_error(e, "large twiddle tables");
+        }
+        g_tables.insert(made.begin(), made.end());
     }
-    const int64_t count = which > 0 ? int64_t(1) << (which - 4) : int64_t(16) << -which;
-    float2 *p = nullptr;
-    e = cudaMalloc(&p, sizeof(float2) * static_cast<size_t>(count));
-    if (e != cudaSuccess) return cuda_error(e, "large twiddle cudaMalloc");
-    cudaStream_t st;
-    e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
-        cudaFree(p);
-        return cuda_error(e, "large twiddle stream");
-    }
-    const unsigned blocks = static_cast<unsigned>((count + 255) / 256);
-    if (which > 0)
-        large_root_kernel<<<blocks, 256, 0, st>>>(p, which, count);
-    else
-        large_stage_kernel<<<blocks, 256, 0, st>>>(p, -which);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    cudaStreamDestroy(st);
-    if (e != cudaSuccess) {
-        cudaFree(p);
-        return cuda_error(e, "large twiddle generation");
-    }
-    g_tables[{dev, which}] = p;
-    *out = p;
+    *root = g_tables[{dev, logn}];
+    *stage = g_tables[{dev, -logn2}];
     return BPLG_OK;
 }
 
@@ -348,8 +352,7 @@ int fft_large_launch(const bplg_plan &p, const void *in, void *out, int64_t n, i
     if (rc != BPLG_OK) return rc;
     int logn = ilog2(n);
     const float2 *root = nullptr, *stage = nullptr;
-    rc = large_table(logn, &root);
-    if (rc == BPLG_OK) rc = large_table(p.n1_log - logn, &stage);
+    rc = large_tables(logn, logn - p.n1_log, &root, &stage);
     if (rc != BPLG_OK) return rc;
     void *y = nullptr;
     rc = stream_scratch(kScratchLargeFft, static_cast<size_t>(n) * static_cast<size_t>(batch) * sizeof(float2), s, &y);

@@ -70,8 +70,8 @@ def test_every_row_count_per_block(bp, row_log):
 
 
 def test_device_memory_of_a_first_call(bp):
-    """One transform of 2^16 points makes its own two tables (64 KB) and its
-    scratch (512 KB), not those of every row length (4 MB)."""
+    """One transform of 2^16 points makes its own tables (290 KB) and its
+    scratch (512 KB), not those of every row length there is (4 MB)."""
     code = """
 import torch, paper_2310_16214_gb300 as bp
 x = torch.zeros(2 << 16, device="cuda")
@@ -86,6 +86,28 @@ print(free - torch.cuda.mem_get_info()[0])
     r = subprocess.run([sys.executable, "-c", code], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0, r.stderr
     assert int(r.stdout) <= 2 << 20
+
+
+def test_any_plan_under_capture_after_one_call(bp):
+    """After a call with an n, a call of any plan of that n can be captured."""
+    n = 1 << 19
+    z = si.fft_c64(1, n, stream=219)
+    zd = c64_to_dev(z)
+    out = torch.empty_like(zd)
+    side = torch.cuda.Stream()
+    plans = {p.n1_log: p for p in bp.enumerate_plans(bp.OP_FFT, bp.F32, n)}
+    with torch.cuda.stream(side):
+        bp.fft_batched(zd, out, n, 1, -1)
+        side.synchronize()
+        ref = oracle.fft(z, -1)
+        for p in plans.values():
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=side):
+                bp.fft_batched(zd, out, n, 1, -1, plan=p)
+            out.zero_()
+            g.replay()
+            side.synchronize()
+            assert fft_rel_err(c64_from_dev(out).reshape(1, n), ref).max() <= 1e-5 * 19, p
 
 
 @pytest.mark.parametrize("logn", [16, 18, 20, 22])
