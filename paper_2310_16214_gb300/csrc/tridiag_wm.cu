@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(MAXT)
 // two blocks of 98 KB fit where one slot a thread takes 118 KB: n = 5000 0.085 ->
 // 0.071 ms; below that it only adds shuffles (0.0594 -> 0.0615 ms at n = 3000).
 //   Measured at 2^24 unknowns, padded power-of-two kernel -> this one: n = 300
-// 0.076 -> 0.062 ms, 700 0.072 -> 0.062, 1500 0.066 -> 0.058, 3000 0.086 -> 0.060 (82
+// 0.076 -> 0.062 ms, 700 0.072 -> 0.062, 1500 0.066 -> 0.055, 3000 0.086 -> 0.060 (82
 // % of the copy bandwidth), 3001 0.182 -> 0.060, 5000 0.124 -> 0.065, 8191 0.195 ->
 // 0.076.
 template <int P, int MAXT, int MINB, bool PER_WARP>
